@@ -52,6 +52,9 @@ cudaError_t launch_rp(const StepArgs& a, unsigned* sync, int W, int R, int NP, i
                       cudaStream_t st);
 int rp_max_ctas(int W, int R, int NP, int JP, int I, long long max_k, int sms);
 size_t rp_smem_bytes(int W, int R, int NP, int JP, long long K);
+// cluster_step.cu
+int rpc_ctas(long long n, int JP);
+cudaError_t launch_rpc(const StepArgs& a, int nspecies, int C, int JP, long long K, cudaStream_t st);
 }  // namespace it
 
 using namespace it;
@@ -603,6 +606,12 @@ int alloc_scratch(iontrap* h) {
 
 // One row-persistent launch of K steps on the handle's buffers.
 cudaError_t launch_rp_of(iontrap* h, const StepArgs& a, long long K, cudaStream_t st) {
+  // steps of a small simulation run on one cluster (same bits); force evaluations, traced
+  // launches and those of the failure test, which look at the grid's counter, do not
+  if (a.mode == MODE_STEP && !a.trace && !a.stall_on && !a.wait_ns) {
+    const int C = rpc_ctas(h->n, h->rp.JP);
+    if (C > 0) return launch_rpc(a, h->nspecies, C, h->rp.JP, K, st);
+  }
   return launch_rp(a, h->d_gsync, h->rp.W, h->rp.R, h->rp.NP, h->rp.JP, h->rp.I, h->rp.G, K, st);
 }
 

@@ -463,6 +463,18 @@ __device__ __forceinline__ void trap_springs(const TrapDev& tp, const SpeciesDev
   k[2] = rwz2;
 }
 
+// Trap spring constant of component c (the c-th value trap_springs gives, same roundings).
+__device__ __forceinline__ double trap_spring_c(const TrapDev& tp, const SpeciesDev& sd, double cosv, int c) {
+  if (tp.flags & IONTRAP_TRAP_OFF) return 0.0;
+  if (tp.flags & IONTRAP_PSEUDO) return sd.ks[c];
+  const double rwz2 = __dmul_rn(sd.rho, tp.wz2);
+  const double rq4 = __dmul_rn(tp.q4, sd.rho);
+  const double qc2 = __dmul_rn(2.0 * tp.q, cosv);
+  const double ax = (c == 0) ? __dsub_rn(tp.a, qc2) : __dadd_rn(tp.a, qc2);
+  const double kr = __fma_rn(rq4, ax, -0.5 * rwz2);
+  return c == 2 ? rwz2 : kr;
+}
+
 // Acceleration of one ion at force time, FP64 in both forms, split in two so that the
 // part that does not depend on the Coulomb sum can be evaluated before the sum is known:
 //   ext = -k xf - gamma vd - lrate (kdir.vd) kdir + sigma xi(seed, counter, id)  (accel_ext)

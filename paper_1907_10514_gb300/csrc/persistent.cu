@@ -68,18 +68,6 @@ __device__ __forceinline__ void arrive_release(unsigned* ctr) {
   asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr) : "memory");
 }
 
-// Trap spring constant of component c (the c-th value trap_springs gives, same roundings).
-__device__ __forceinline__ double trap_spring_c(const TrapDev& tp, const SpeciesDev& sd, double cosv, int c) {
-  if (tp.flags & IONTRAP_TRAP_OFF) return 0.0;
-  if (tp.flags & IONTRAP_PSEUDO) return sd.ks[c];
-  const double rwz2 = __dmul_rn(sd.rho, tp.wz2);
-  const double rq4 = __dmul_rn(tp.q4, sd.rho);
-  const double qc2 = __dmul_rn(2.0 * tp.q, cosv);
-  const double ax = (c == 0) ? __dsub_rn(tp.a, qc2) : __dadd_rn(tp.a, qc2);
-  const double kr = __fma_rn(rq4, ax, -0.5 * rwz2);
-  return c == 2 ? rwz2 : kr;
-}
-
 template <int W>
 __global__ void __launch_bounds__(32 * W, 16 / W) k_step_f32_gp(const __grid_constant__ StepArgs A, const GpArgs P) {
   constexpr int T = 32 * W;
