@@ -348,7 +348,11 @@ typedef struct {
                                     IONTRAP_COULOMB_OFF.
                                  Form 5 gives results within the FP32 tolerances of the other
                                  forms, bitwise reproducible for a given shape.
-                                 The FP64 form supports 1 only. */
+                                 Up to 432 ions form 5 steps run on one thread-block
+                                 cluster instead, with the same bits.
+                                 The FP64 form supports 1 only; it sums every unordered pair
+                                 once in a layout that is a function of n, and threads,
+                                 ions_per_thread and jsplit do not change its results. */
     int32_t pdl;              /* 1: consecutive step kernels use programmatic dependent launch
                                  (default 0: measured slower on GB300 for these grids) */
     int32_t graph;            /* 1: iontrap_step enqueues CUDA graphs of 100 steps; 0: single launches */

@@ -27,7 +27,7 @@
 #include "iontrap_internal.cuh"
 
 namespace it {
-const void* step_kernel(int f64, int T, int I, int packed, int fused);
+const void* step_kernel(int T, int I, int packed, int fused);
 const void* prep_kernel();
 }  // namespace it
 
@@ -136,7 +136,7 @@ extern "C" int iontrap_forces_noalloc(const iontrap_species* species, int n_spec
   if (e == cudaSuccess) e = cudaLaunchKernel(prep_kernel(), dim3(prep_blocks), dim3(256), prep_params, 0, stream);
   void* params[] = {&A};
   if (e == cudaSuccess)
-    e = cudaLaunchKernel(step_kernel(0, kNoAllocThreads, 1, 0, 1), dim3((unsigned)iblocks, (unsigned)A.nsplit),
+    e = cudaLaunchKernel(step_kernel(kNoAllocThreads, 1, 0, 1), dim3((unsigned)iblocks, (unsigned)A.nsplit),
                          dim3(kNoAllocThreads), params, 0, stream);
   return e == cudaSuccess ? IONTRAP_OK : IONTRAP_ECUDA;
 }

@@ -26,8 +26,8 @@ int batched_max_n();
 bool batched_shape_fits(long long n, int C, int NP);
 cudaError_t launch_batched(const std::vector<BatchEns>& ens, const std::vector<long long>& steps, int K,
                            cudaStream_t stream);
-const void* step_kernel(int f64, int T, int I, int packed, int fused);
-const void* epilogue_kernel(int f64);
+const void* step_kernel(int T, int I, int packed, int fused);
+const void* epilogue_kernel();
 cudaError_t allow_large_clusters();
 const void* prep_kernel();
 const void* restore_kernel();
@@ -52,6 +52,10 @@ cudaError_t launch_rp(const StepArgs& a, unsigned* sync, int W, int R, int NP, i
                       cudaStream_t st);
 int rp_max_ctas(int W, int R, int NP, int JP, int I, long long max_k, int sms);
 size_t rp_smem_bytes(int W, int R, int NP, int JP, long long K);
+// pairs_f64.cu
+size_t f64_scratch_bytes(long long n, int sms);
+cudaError_t f64_prepare(long long n, int sms, void* scratch, cudaStream_t st, F64View* v);
+cudaError_t launch_f64(const StepArgs& a, const F64View& v, int nspecies, cudaStream_t st);
 // cluster_step.cu
 int rpc_ctas(long long n, int JP);
 cudaError_t launch_rpc(const StepArgs& a, int nspecies, int C, int JP, long long K, cudaStream_t st);
@@ -60,7 +64,7 @@ cudaError_t launch_rpc(const StepArgs& a, int nspecies, int C, int JP, long long
 using namespace it;
 
 static constexpr int kGraphSteps = 100;
-static constexpr int kMaxJsplitF64 = 2048;  // FP64 form stages its whole j-range
+static constexpr int kMaxJsplitF64 = 2048;  // largest jsplit an FP64 configuration may name
 static constexpr int64_t kMaxSplitsUnfused = 64;
 static constexpr int64_t kMaxClusterSplits = 8;   // portable cluster size (form 2)
 static constexpr int64_t kMaxClusterSplits3 = 16; // non-portable cluster size (form 3)
@@ -115,6 +119,7 @@ struct iontrap {
   int T = 128, I = 1, packed = 0, jsplit = 128, fused = 1, pdl = 0, use_graph = 1;
   GpShape gp{};                 // fused = 4
   RpShape rp{};                 // fused = 5
+  F64View f64v{};               // FP64 form: its scratch
   unsigned* d_gsync = nullptr;  // fused = 4, 5: step and group counters (zero between launches)
   double* d_snap = nullptr;     // iontrap_step_record: x_{s-W}, x_{s-W+1} [2][3][n]
   StepArgs args{};
@@ -140,6 +145,13 @@ struct DeviceGuard {
 };
 
 int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
+
+// Whether a form 0 .. 3 configuration exists.  The FP64 form lays its work out by itself: it
+// accepts these shapes (and a jsplit) and computes the same bits with each.
+bool form_exists(int f64, int T, int I, int packed, int fused) {
+  if (!f64) return step_kernel(T, I, packed, fused) != nullptr;
+  return fused == 1 && packed == 0 && ((I == 1 && (T == 64 || T == 128 || T == 256)) || (I == 2 && T == 128));
+}
 
 // Shape of a grid-persistent configuration (FP32 form with the pair term, 256 or 512
 // threads, two ions per lane packed, at least seven segments, every CTA co-resident),
@@ -468,11 +480,6 @@ dim3 grid_of(const iontrap* h) {
   return dim3((unsigned)cdiv(h->n, iblock_ions(h)), (unsigned)splits_of(h), 1);
 }
 
-size_t smem_of(const iontrap* h) {
-  if (!h->f64 || (h->p.flags & IONTRAP_COULOMB_OFF)) return 0;  // FP32 form: static chunk buffers
-  return (size_t)h->jsplit * 32;
-}
-
 // The per-species constants and the trap of a handle's step arguments, from the trap and
 // default bath of p and, when cool is not null, one bath and laser per species.
 void fill_forces(iontrap* h, const iontrap_params* p, const iontrap_cooling* cool) {
@@ -565,9 +572,9 @@ int alloc_scratch(iontrap* h) {
   if (h->fused == 5 &&
       !rp_shape(h->n, h->f64, h->p.flags, h->sms, h->T, h->I, h->packed, h->jsplit, &h->rp))
     return IONTRAP_EINVAL;
-  // one 32-byte record per (split, ion) in both forms; the row-persistent form also keeps
+  // FP32 form: one 32-byte record per (split, ion); the row-persistent form also keeps
   // its part-major position copies there between the steps of a launch
-  size_t part = (size_t)splits * (size_t)h->n * 32;
+  size_t part = h->f64 ? f64_scratch_bytes(h->n, h->sms) : (size_t)splits * (size_t)h->n * 32;
   if (h->fused == 5) part = std::max(part, rp_scratch_bytes(h->rp.NP, h->rp.JP));
   const size_t cnt = (size_t)cdiv(h->n, iblock_ions(h));
   if (part > h->part_bytes) {
@@ -595,6 +602,7 @@ int alloc_scratch(iontrap* h) {
       if (cudaMemsetAsync(h->d_gsync, 0, kGpSyncBytes, h->stream) != cudaSuccess) return IONTRAP_ECUDA;
     }
   }
+  if (h->f64 && f64_prepare(h->n, h->sms, h->d_part, h->stream, &h->f64v) != cudaSuccess) return IONTRAP_ECUDA;
   h->args.part = h->d_part;
   h->args.cnt = h->d_cnt;
   h->args.jsplit = (h->p.flags & IONTRAP_COULOMB_OFF) ? (int)std::min<int64_t>(h->n, 1 << 30)
@@ -618,6 +626,7 @@ cudaError_t launch_rp_of(iontrap* h, const StepArgs& a, long long K, cudaStream_
 // Launch one step kernel with programmatic dependent launch, so that consecutive steps
 // overlap one grid's launch with the previous grid's tail.
 cudaError_t launch_step_on(iontrap* h, StepArgs& a, cudaStream_t st) {
+  if (h->f64) return launch_f64(a, h->f64v, h->nspecies, st);
   if (h->fused == 5 && a.mode != MODE_INIT)
     return launch_rp_of(h, a, 1, st);
   if (h->fused == 4 || h->fused == 5) {
@@ -629,12 +638,11 @@ cudaError_t launch_step_on(iontrap* h, StepArgs& a, cudaStream_t st) {
     cfg.blockDim = dim3(128);
     cfg.stream = st;
     void* params[] = {&a};
-    return cudaLaunchKernelExC(&cfg, step_kernel(0, 128, 2, 1, 1), params);
+    return cudaLaunchKernelExC(&cfg, step_kernel(128, 2, 1, 1), params);
   }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid_of(h);
   cfg.blockDim = dim3(h->T);
-  cfg.dynamicSmemBytes = smem_of(h);
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   int na = 0;
@@ -653,12 +661,12 @@ cudaError_t launch_step_on(iontrap* h, StepArgs& a, cudaStream_t st) {
   cfg.attrs = attr;
   cfg.numAttrs = na;
   void* params[] = {&a};
-  cudaError_t e = cudaLaunchKernelExC(&cfg, step_kernel(h->f64, h->T, h->I, h->packed, h->fused), params);
+  cudaError_t e = cudaLaunchKernelExC(&cfg, step_kernel(h->T, h->I, h->packed, h->fused), params);
   if (e != cudaSuccess || h->fused != 0) return e;
   cfg.gridDim = dim3((unsigned)cdiv(h->n, 32));  // 32 ions per epilogue CTA
   cfg.blockDim = dim3(256);
   cfg.dynamicSmemBytes = 0;
-  return cudaLaunchKernelExC(&cfg, epilogue_kernel(h->f64), params);
+  return cudaLaunchKernelExC(&cfg, epilogue_kernel(), params);
 }
 
 cudaError_t launch_mode(iontrap* h, int mode, double* out) {
@@ -710,15 +718,6 @@ cudaError_t build_graph(iontrap* h) {
 int prepare_kernels() {
   static int done = 0;
   if (done) return IONTRAP_OK;
-  const int Ts[] = {64, 128, 256};
-  const int Is[] = {1, 2, 4};
-  for (int T : Ts)
-    for (int I : Is) {
-      const void* fn = step_kernel(1, T, I, 0, 1);
-      if (fn && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxJsplitF64 * 32) !=
-                    cudaSuccess)
-        return IONTRAP_ECUDA;
-    }
   if (allow_large_clusters() != cudaSuccess) return IONTRAP_ECUDA;
   done = 1;
   return IONTRAP_OK;
@@ -885,7 +884,7 @@ int iontrap_create(const iontrap_species* species, int n_species, const uint8_t*
         h->T = tc.threads, h->I = tc.ions_per_thread, h->packed = tc.packed, h->jsplit = tc.jsplit;
         h->fused = 5, h->pdl = 0, h->use_graph = 0;
       }
-    } else if (tuned && step_kernel(h->f64, tc.threads, tc.ions_per_thread, tc.packed, tc.fused) &&
+    } else if (tuned && form_exists(h->f64, tc.threads, tc.ions_per_thread, tc.packed, tc.fused) &&
         tc.jsplit >= 1 && tc.jsplit <= n && (!h->f64 || tc.jsplit <= kMaxJsplitF64) &&
         (tc.fused || cdiv(n, tc.jsplit) <= kMaxSplitsUnfused) &&
         (tc.fused < 2 || (cdiv(n, tc.jsplit) <= (tc.fused == 3 ? kMaxClusterSplits3 : kMaxClusterSplits) &&
@@ -1451,13 +1450,13 @@ int iontrap_estimate_bytes(int64_t n, int precision, int64_t* bytes) {
   GpShape gs;
   RpShape rs;
   if (tuned_config(n, f64, dev, &tc) &&
-      (step_kernel(f64, tc.threads, tc.ions_per_thread, tc.packed, tc.fused) ||
+      (form_exists(f64, tc.threads, tc.ions_per_thread, tc.packed, tc.fused) ||
        (tc.fused == 4 && gp_shape(n, f64, 0, sms, tc.threads, tc.ions_per_thread, tc.packed, tc.jsplit, &gs)) ||
        (tc.fused == 5 && rp_shape(n, f64, 0, sms, tc.threads, tc.ions_per_thread, tc.packed, tc.jsplit, &rs)))) {
     T = tc.threads, I = tc.ions_per_thread, J = tc.jsplit, F = tc.fused;
   }
   const int64_t splits = F == 5 ? cdiv(n, kRpInitJsplit) : cdiv(n, J);
-  int64_t part = splits * n * 32;
+  int64_t part = f64 ? (int64_t)f64_scratch_bytes(n, sms) : splits * n * 32;
   if (F == 5 && rp_shape(n, f64, 0, sms, T, I, P, J, &rs))
     part = std::max<int64_t>(part, (int64_t)rp_scratch_bytes(rs.NP, rs.JP));
   const int64_t iblocks = F >= 4 ? cdiv(n, 256) : cdiv(n, (F == 3 ? 32 : (int64_t)T) * I);
@@ -1484,9 +1483,7 @@ int iontrap_autotune(iontrap_t* h, double trial_us, iontrap_config* best, double
     int T, I, P;
   };
   std::vector<Shape> shapes;
-  if (h->f64) {
-    shapes = {{64, 1, 0}, {128, 1, 0}, {128, 2, 0}, {256, 1, 0}};
-  } else {
+  if (!h->f64) {
     const Shape small[] = {{32, 1, 0}, {64, 1, 0}, {128, 1, 0}, {64, 2, 1}, {128, 2, 1}};
     const Shape large[] = {{64, 4, 1}, {128, 4, 1}, {256, 4, 1}, {128, 2, 1}};
     if (n < 16384) {
@@ -1497,6 +1494,7 @@ int iontrap_autotune(iontrap_t* h, double trial_us, iontrap_config* best, double
     }
   }
   std::vector<iontrap_config> cands;
+  if (h->f64) cands.push_back(orig);  // the FP64 form has one layout
   for (const Shape& sh : shapes) {
     const int64_t iblocks = cdiv(n, (int64_t)sh.T * sh.I);
     std::vector<int64_t> splits = {1, 2, 3, 4, 6, 8};
@@ -1509,14 +1507,13 @@ int iontrap_autotune(iontrap_t* h, double trial_us, iontrap_config* best, double
     std::sort(splits.begin(), splits.end());
     splits.erase(std::unique(splits.begin(), splits.end()), splits.end());
     for (int64_t S : splits) {
-      if (S < 1 || S > 64 || S > std::max<int64_t>(1, n / (h->f64 ? 8 : 32))) continue;
+      if (S < 1 || S > 64 || S > std::max<int64_t>(1, n / 32)) continue;
       int64_t js = cdiv(n, S);
-      if (h->f64 && js > kMaxJsplitF64) continue;
-      for (int fused = 2; fused >= (h->f64 ? 1 : 0); --fused) {
-        if (fused == 2 && (h->f64 || cdiv(n, js) > kMaxClusterSplits || (h->p.flags & IONTRAP_COULOMB_OFF))) continue;
+      for (int fused = 2; fused >= 0; --fused) {
+        if (fused == 2 && (cdiv(n, js) > kMaxClusterSplits || (h->p.flags & IONTRAP_COULOMB_OFF))) continue;
         if (!fused && cdiv(n, js) > kMaxSplitsUnfused) continue;
         iontrap_config c{sh.T, sh.I, sh.P, (int32_t)js, fused, 0, 1};
-        if (step_kernel(h->f64, c.threads, c.ions_per_thread, c.packed, c.fused)) cands.push_back(c);
+        if (step_kernel(c.threads, c.ions_per_thread, c.packed, c.fused)) cands.push_back(c);
       }
     }
   }
@@ -1526,7 +1523,7 @@ int iontrap_autotune(iontrap_t* h, double trial_us, iontrap_config* best, double
       for (int64_t S = 2; S <= kMaxClusterSplits3; S *= 2) {
         if (S > std::max<int64_t>(1, n / 128)) continue;
         iontrap_config c{32 * iw[1], iw[0], iw[0] == 2 ? 1 : 0, (int32_t)cdiv(n, S), 3, 0, 1};
-        if (step_kernel(0, c.threads, c.ions_per_thread, c.packed, 3)) cands.push_back(c);
+        if (step_kernel(c.threads, c.ions_per_thread, c.packed, 3)) cands.push_back(c);
       }
   }
   if (!h->f64 && !(h->p.flags & IONTRAP_COULOMB_OFF)) {  // grid-persistent shapes: one or two CTAs per SM
@@ -1797,7 +1794,7 @@ int iontrap_set_config(iontrap_t* h, const iontrap_config* c) {
   } else if (c->fused == 5) {
     if (!rp_shape(h->n, h->f64, h->p.flags, h->sms, c->threads, c->ions_per_thread, c->packed, c->jsplit, &rs))
       return IONTRAP_EINVAL;
-  } else if (!step_kernel(h->f64, c->threads, c->ions_per_thread, c->packed, c->fused)) {
+  } else if (!form_exists(h->f64, c->threads, c->ions_per_thread, c->packed, c->fused)) {
     return IONTRAP_EINVAL;
   }
   if (c->jsplit < 1 || c->jsplit > h->n || (h->f64 && c->jsplit > kMaxJsplitF64)) return IONTRAP_EINVAL;

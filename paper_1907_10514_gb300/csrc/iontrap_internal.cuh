@@ -101,6 +101,14 @@ struct BatchEns {
   SpeciesDev spc[IONTRAP_MAX_SPECIES];
 };
 
+// Scratch of an FP64 handle (pairs_f64.cu): its tables and slots, by offset from base, and the
+// shape of its pair line.
+struct F64View {
+  void* base;
+  size_t off[9];
+  int I, rows, cols, warps;
+};
+
 // ------------------------------------------------------------------ PTX helpers
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {

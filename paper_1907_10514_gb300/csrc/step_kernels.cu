@@ -30,29 +30,6 @@ namespace it {
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// Stage a whole j-range (bytes per stream) with bulk TMA; every thread waits with a
-// time limit.  Returns false (error flag set, copies drained) if the wait expired.
-__device__ __forceinline__ bool stage_jrange(uint64_t* bar, void* d0, const void* s0, void* d1, const void* s1,
-                                             uint32_t bytes, int* err) {
-  if (threadIdx.x == 0) mbar_init(bar, 1);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    mbar_arrive_expect_tx(bar, s1 ? 2u * bytes : bytes);
-    tma_bulk_g2s(d0, s0, bytes, bar);
-    if (s1) tma_bulk_g2s(d1, s1, bytes, bar);
-  }
-  const bool ok = mbar_wait_bounded(bar, 0, kWaitLimitNs);
-  if (__syncthreads_or(!ok)) {
-    if (threadIdx.x == 0) {
-      atomicOr(err, ERR_TIMEOUT);
-      mbar_wait_bounded(bar, 0, kWaitLimitNs);
-    }
-    __syncthreads();
-    return false;
-  }
-  return true;
-}
-
 // Arrival at the i-block counter; true in the last CTA of the i-block.
 __device__ __forceinline__ bool arrive_last(unsigned* cnt, unsigned expected, int* s_flag) {
   __threadfence();
@@ -80,19 +57,6 @@ __device__ __forceinline__ void finish_iblock(const StepArgs& A, long long ns) {
       __threadfence();
     }
   }
-}
-
-__device__ __forceinline__ void merge_f64(const double4_32a* __restrict__ part, long long n, long long i,
-                                          int nsplit, double S[3]) {
-  double s[3] = {0.0, 0.0, 0.0};
-  for (int p = 0; p < nsplit; ++p) {
-    const double2* r = reinterpret_cast<const double2*>(part + p * n + i);
-    const double2 xy = __ldcg(r), zw = __ldcg(r + 1);
-    s[0] += xy.x;
-    s[1] += xy.y;
-    s[2] += zw.x;
-  }
-  S[0] = s[0], S[1] = s[1], S[2] = s[2];
 }
 
 // ------------------------------------------------------------------ FP32 form
@@ -721,107 +685,6 @@ __global__ void __launch_bounds__(kEpiThreads) k_epilogue_f32(const __grid_const
   trace_mark(et, 2ll * blockIdx.x + 1);
 }
 
-// ------------------------------------------------------------------ FP64 plain form
-template <int I, bool DIAG>
-__device__ __forceinline__ void segment_f64(const double4_32a* __restrict__ sp, int g0, int g1, long long jbase,
-                                            const double (&xi)[I][3], const long long (&ii)[I],
-                                            double (&acc)[I][3]) {
-#pragma unroll 2
-  for (int j = g0; j < g1; ++j) {
-    const double4_32a p = sp[j];
-#pragma unroll
-    for (int k = 0; k < I; ++k) {
-      const double dx = xi[k][0] - p.x;
-      const double dy = xi[k][1] - p.y;
-      const double dz = xi[k][2] - p.z;
-      const double r2 = dx * dx + dy * dy + dz * dz;
-      double ri = rsqrt(r2);
-      if (DIAG) ri = (jbase + j == ii[k]) ? 0.0 : ri;
-      const double s = p.w * ri * ri * ri;
-      acc[k][0] += s * dx;
-      acc[k][1] += s * dy;
-      acc[k][2] += s * dz;
-    }
-  }
-}
-
-template <int T, int I>
-__global__ void __launch_bounds__(T) k_step_f64(const __grid_constant__ StepArgs A) {
-  extern __shared__ __align__(128) unsigned char smraw[];
-  __shared__ __align__(8) uint64_t bar;
-  __shared__ int s_flag;
-  __shared__ double s_cos;
-  double4_32a* sp = reinterpret_cast<double4_32a*>(smraw);
-  __shared__ double s_springs[IONTRAP_MAX_SPECIES][3];
-
-  pdl_wait();
-  const int tid = threadIdx.x;
-  const long long n = A.n;
-  const long long i0 = (long long)blockIdx.x * (T * I);
-  const long long j0 = (long long)blockIdx.y * A.jsplit;
-  const int jn = (int)min((long long)A.jsplit, n - j0);  // FP64 form: whole j-range staged
-  const long long ns = *A.step;
-  const int rb = (A.mode == MODE_STEP) ? (int)((ns + 1) & 1) : (int)(ns & 1);
-  const bool coulomb = !(A.trap.flags & IONTRAP_COULOMB_OFF);
-
-  double acc[I][3];
-#pragma unroll
-  for (int k = 0; k < I; ++k)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) acc[k][c] = 0.0;
-
-  if (coulomb) {
-    if (!stage_jrange(&bar, sp, A.p64[rb] + j0, nullptr, nullptr, (uint32_t)jn * 32u, A.err)) return;
-    double xi[I][3];
-    long long ii[I];
-#pragma unroll
-    for (int k = 0; k < I; ++k) {
-      ii[k] = i0 + k * T + tid;
-      double4_32a p = make_double4_32a(0., 0., 0., 0.);
-      if (ii[k] < n) p = A.p64[rb][ii[k]];
-      xi[k][0] = p.x, xi[k][1] = p.y, xi[k][2] = p.z;
-    }
-    const long long iend = i0 + T * I;
-    for (int g0 = 0; g0 < jn; g0 += kSeg) {
-      const int g1 = min(g0 + kSeg, jn);
-      const bool diag = (j0 + g0 < iend) && (i0 < j0 + g1);
-      if (diag)
-        segment_f64<I, true>(sp, g0, g1, j0, xi, ii, acc);
-      else
-        segment_f64<I, false>(sp, g0, g1, j0, xi, ii, acc);
-    }
-  }
-
-  pdl_trigger();
-  double4_32a* part = reinterpret_cast<double4_32a*>(A.part);
-#pragma unroll
-  for (int k = 0; k < I; ++k) {
-    const long long i = i0 + k * T + tid;
-    if (i < n) {
-      double2* r = reinterpret_cast<double2*>(part + blockIdx.y * n + i);
-      __stcg(r, make_double2(acc[k][0], acc[k][1]));
-      __stcg(r + 1, make_double2(acc[k][2], 0.0));
-    }
-  }
-  if (!arrive_last(&A.cnt[blockIdx.x], gridDim.y, &s_flag)) return;
-
-  if (tid == 0) s_cos = force_time_cos(A, ns);
-  __syncthreads();
-  if (tid < IONTRAP_MAX_SPECIES) trap_springs(A.trap, A.spc[tid], s_cos, s_springs[tid]);
-  __syncthreads();
-  const int wb = rb ^ 1;
-  const int nsplit = gridDim.y;
-#pragma unroll
-  for (int k = 0; k < I; ++k) {
-    const long long i = i0 + k * T + tid;
-    if (i >= n) continue;
-    double S[3];
-    merge_f64(part, n, i, nsplit, S);
-    epilogue_ion<true>(A, i, S, s_springs, ns, wb);
-  }
-  finish_iblock(A, ns);
-}
-
 // ------------------------------------------------------------------ helpers
 // Write pair stream b from the FP64 positions x_n (create and force evaluation).
 __global__ void k_prep(const __grid_constant__ StepArgs A, int b, int f64) {
@@ -872,14 +735,14 @@ __global__ void k_normals(unsigned long long seed, long long counter, const long
 
 // ------------------------------------------------------------------ registry
 struct KernelEntry {
-  int f64, T, I, packed, fused;
+  int T, I, packed, fused;
   const void* fn;
 };
 
-#define IT_F32(T, I, P) {0, T, I, P, 1, (const void*)k_step_f32<T, I, P, true>}, \
-                        {0, T, I, P, 0, (const void*)k_step_f32<T, I, P, false>}, \
-                        {0, T, I, P, 2, (const void*)k_step_f32_cl<T, I, P>}
-#define IT_CW(I, W, P) {0, 32 * W, I, P, 3, (const void*)k_step_f32_cw<I, W, P>}
+#define IT_F32(T, I, P) {T, I, P, 1, (const void*)k_step_f32<T, I, P, true>}, \
+                        {T, I, P, 0, (const void*)k_step_f32<T, I, P, false>}, \
+                        {T, I, P, 2, (const void*)k_step_f32_cl<T, I, P>}
+#define IT_CW(I, W, P) {32 * W, I, P, 3, (const void*)k_step_f32_cw<I, W, P>}
 static const KernelEntry kKernels[] = {
     IT_CW(1, 2, false), IT_CW(1, 4, false), IT_CW(2, 2, true), IT_CW(2, 4, true),
     IT_F32(32, 1, false),  IT_F32(32, 2, true),
@@ -887,15 +750,13 @@ static const KernelEntry kKernels[] = {
     IT_F32(128, 1, false), IT_F32(128, 2, false), IT_F32(128, 2, true), IT_F32(128, 4, false),
     IT_F32(128, 4, true),  IT_F32(256, 1, false), IT_F32(256, 2, true), IT_F32(256, 4, true),
     IT_F32(256, 4, false),
-    {1, 64, 1, 0, 1, (const void*)k_step_f64<64, 1>},   {1, 128, 1, 0, 1, (const void*)k_step_f64<128, 1>},
-    {1, 128, 2, 0, 1, (const void*)k_step_f64<128, 2>}, {1, 256, 1, 0, 1, (const void*)k_step_f64<256, 1>},
 };
 #undef IT_F32
 #undef IT_CW
 
-const void* step_kernel(int f64, int T, int I, int packed, int fused) {
+const void* step_kernel(int T, int I, int packed, int fused) {
   for (const auto& e : kKernels)
-    if (e.f64 == f64 && e.T == T && e.I == I && e.packed == packed && e.fused == fused) return e.fn;
+    if (e.T == T && e.I == I && e.packed == packed && e.fused == fused) return e.fn;
   return nullptr;
 }
 
@@ -909,7 +770,7 @@ cudaError_t allow_large_clusters() {
   return cudaSuccess;
 }
 
-const void* epilogue_kernel(int f64) { return f64 ? nullptr : (const void*)k_epilogue_f32; }
+const void* epilogue_kernel() { return (const void*)k_epilogue_f32; }
 
 const void* prep_kernel() { return (const void*)k_prep; }
 const void* restore_kernel() { return (const void*)k_restore; }
