@@ -73,38 +73,6 @@ __device__ __forceinline__ void bar_arrive(int id, int threads) {
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
-// (double)x without the FP64-rate conversion: normal floats and zeros by their bits.
-__device__ __forceinline__ double widen(float x) {
-  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
-  if (m - 0x00800000u < 0x7f000000u)  // normal
-    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
-  if (m == 0u) return __hiloint2double((int)b, 0);
-  return (double)x;
-}
-
-// hi = fl(x), lo = fl(x - hi) without FP64-rate operations: the mantissa's top 24 bits
-// rounded to nearest even, the signed remainder converted and scaled (exact but for its own
-// rounding).  Exponents outside the range where hi and lo are both normal take the plain way.
-__device__ __forceinline__ void split_hilo(double x, float& hi, float& lo) {
-  const unsigned xh = (unsigned)__double2hiint(x), xl = (unsigned)__double2loint(x);
-  const unsigned e = (xh >> 20) & 0x7ffu;
-  if (e - 960u <= 180u) {
-    const unsigned m = ((xh & 0xfffffu) << 3) | (xl >> 29), rem = xl & 0x1fffffffu;
-    const unsigned up = (rem + (m & 1u) > 0x10000000u) ? 1u : 0u;
-    hi = __uint_as_float((xh & 0x80000000u) | (((e - 896u) << 23) + m + up));
-    const int r = (int)rem - (int)(up << 29);
-    lo = __int2float_rn((xh >> 31) ? -r : r) * __uint_as_float((e - 948u) << 23);
-    return;
-  }
-  hi = __double2float_rn(x);
-  lo = __double2float_rn(x - (double)hi);
-}
-
-// Positions are kept as records of four ions: rows x, y, z hi and x, y, z lo of four floats
-// (96 bytes), so one address and constant offsets reach all of a record.  Float of ion e, row r:
-constexpr int kRpcRec = 24;
-__device__ __forceinline__ int rpc_at(int e, int r) { return (e >> 2) * kRpcRec + 4 * r + (e & 3); }
-
 // Part sums are kept [part][kRpcOwners] by owner thread: constant offsets for the merge.
 
 // The sums of one ion (global index i) against the parts first, first + G, ... below NPe, left
@@ -124,25 +92,10 @@ __device__ __forceinline__ void rpc_parts(const float* sb, const float* wz, floa
   for (int g = 0; g < groups; ++g) {
     for (int k = 0; k < per; ++k, p += G)
       if (p < NPe) {
-        float2 acc[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-        const int j0 = p * JP;
-        const float4* rec = reinterpret_cast<const float4*>(sb + rpc_at(j0, 0));
-        const float4* sw = reinterpret_cast<const float4*>(wz + j0);
-#pragma unroll 2
-        for (int q = 0; q < JP; q += 4, rec += kRpcRec / 4) {
-          const float4 hx = rec[0], hy = rec[1], hz = rec[2], lx = rec[3], ly = rec[4], lz = rec[5];
-          float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (!UNITW) w = sw[q >> 2];
-          rp_pair2<true, UNITW>(make_float2(hx.x, hx.y), make_float2(hy.x, hy.y), make_float2(hz.x, hz.y),
-                                make_float2(lx.x, lx.y), make_float2(ly.x, ly.y), make_float2(lz.x, lz.y),
-                                make_float2(w.x, w.y), j0 + q, i, nh, nl, acc);
-          rp_pair2<true, UNITW>(make_float2(hx.z, hx.w), make_float2(hy.z, hy.w), make_float2(hz.z, hz.w),
-                                make_float2(lx.z, lx.w), make_float2(ly.z, ly.w), make_float2(lz.z, lz.w),
-                                make_float2(w.z, w.w), j0 + q + 2, i, nh, nl, acc);
-        }
-        // a part is one chunk: its Kahan sum is 0 + (even + odd), without compensation
+        float f[3];
+        rec_part<UNITW>(sb, wz, p * JP, JP, i, nh, nl, f);
 #pragma unroll
-        for (int d = 0; d < 3; ++d) ps[p * kRpcOwners + d * row] = 0.0f + (acc[d].x + acc[d].y);
+        for (int d = 0; d < 3; ++d) ps[p * kRpcOwners + d * row] = f[d];
       }
     bar_arrive(1 + g, kRpcOwners + kRpcPairs);
   }

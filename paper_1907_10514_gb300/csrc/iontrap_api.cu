@@ -52,6 +52,12 @@ cudaError_t launch_rp(const StepArgs& a, unsigned* sync, int W, int R, int NP, i
                       cudaStream_t st);
 int rp_max_ctas(int W, int R, int NP, int JP, int I, long long max_k, int sms);
 size_t rp_smem_bytes(int W, int R, int NP, int JP, long long K);
+// minimize.cu
+bool minimize_shape(long long n, int R, int NP, int JP, int sms, int* ctas, int* ions, bool* cluster);
+size_t minimize_scratch_bytes(long long n, int ctas);
+cudaError_t launch_minimize(const StepArgs& s, void* scratch, bool cluster, int ctas, int ions, int NP, int JP,
+                            double dt, double dmax, double ftol, long long iters, int final_eval, int b,
+                            cudaStream_t st);
 // pairs_f64.cu
 size_t f64_scratch_bytes(long long n, int sms);
 cudaError_t f64_prepare(long long n, int sms, void* scratch, cudaStream_t st, F64View* v);
@@ -1078,52 +1084,80 @@ int iontrap_minimize(iontrap_t* h, int64_t max_iters, double dt, double dmax, do
   if (st) return st;
   DeviceGuard g(h->device);
   const size_t vec = 3 * (size_t)h->n * sizeof(double);
-  if (!h->d_out && dev_alloc(h, &h->d_out, vec) != cudaSuccess) return IONTRAP_ENOMEM;
-  void* scratch = nullptr;
-  if (cudaMalloc(&scratch, min_scratch_bytes(h->n)) != cudaSuccess) return IONTRAP_ENOMEM;
   const double step_dt = dt > 0 ? dt : h->p.dt;
   const int b = (int)(h->step & 1);  // the pair stream of parity n holds x_n
-  std::vector<unsigned char> hs(min_state_bytes());
   long long done = 0;
   double fn = 0.0;
-  int conv = 0;
-  cudaError_t e = cudaMemsetAsync(scratch, 0, min_scratch_bytes(h->n), h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->d_v, 0, vec, h->stream);  // from rest
-  if (e == cudaSuccess && (h->p.flags & IONTRAP_COULOMB_OFF)) e = cudaMemsetAsync(h->d_out, 0, vec, h->stream);
-  if (e == cudaSuccess) e = launch_prep(h, b);
-  constexpr int64_t kChunk = 64;
-  for (int64_t launched = 0; e == cudaSuccess && launched < max_iters;) {
-    // up to kChunk iterations, then a look at the device state
-    const int64_t k = std::min<int64_t>(kChunk, max_iters - launched);
-    for (int64_t q = 0; q < k && e == cudaSuccess; ++q) {
+  cudaError_t e = cudaSuccess;
+  int ctas = 0, ions = 0;
+  bool cluster = false;
+  if (h->fused == 5 && minimize_shape(h->n, h->rp.R, h->rp.NP, h->rp.JP, h->sms, &ctas, &ions, &cluster)) {
+    // the iterations in launches of at most kGpMaxSteps, a look at the result after each
+    void* scratch = nullptr;
+    const size_t bytes = minimize_scratch_bytes(h->n, ctas);
+    if (dev_alloc(h, &scratch, bytes) != cudaSuccess) return IONTRAP_ENOMEM;
+    MinResult r{};
+    e = cudaMemsetAsync(scratch, 0, bytes, h->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->d_v, 0, vec, h->stream);  // from rest
+    if (e == cudaSuccess) e = launch_prep(h, b);
+    for (int64_t launched = 0; e == cudaSuccess;) {
+      const int64_t k = std::min<int64_t>(kGpMaxSteps, max_iters - launched);
+      launched += k;
+      e = launch_minimize(h->args, scratch, cluster, ctas, ions, h->rp.NP, h->rp.JP, step_dt, dmax, ftol, k,
+                          launched == max_iters, b, h->stream);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(&r, scratch, sizeof(r), cudaMemcpyDeviceToHost, h->stream);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+      if (r.converged || launched == max_iters) break;
+    }
+    dev_free(h, scratch);
+    done = r.iters, fn = r.fnorm;
+    if (e != cudaSuccess) return cuda_status(h, e);
+    st = iontrap_sync(h);  // a wait that gave up
+    if (st) return st;
+  } else {
+    if (!h->d_out && dev_alloc(h, &h->d_out, vec) != cudaSuccess) return IONTRAP_ENOMEM;
+    void* scratch = nullptr;
+    if (cudaMalloc(&scratch, min_scratch_bytes(h->n)) != cudaSuccess) return IONTRAP_ENOMEM;
+    std::vector<unsigned char> hs(min_state_bytes());
+    int conv = 0;
+    e = cudaMemsetAsync(scratch, 0, min_scratch_bytes(h->n), h->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->d_v, 0, vec, h->stream);  // from rest
+    if (e == cudaSuccess && (h->p.flags & IONTRAP_COULOMB_OFF)) e = cudaMemsetAsync(h->d_out, 0, vec, h->stream);
+    if (e == cudaSuccess) e = launch_prep(h, b);
+    constexpr int64_t kChunk = 64;
+    for (int64_t launched = 0; e == cudaSuccess && launched < max_iters;) {
+      // up to kChunk iterations, then a look at the device state
+      const int64_t k = std::min<int64_t>(kChunk, max_iters - launched);
+      for (int64_t q = 0; q < k && e == cudaSuccess; ++q) {
+        if (!(h->p.flags & IONTRAP_COULOMB_OFF)) e = launch_mode(h, MODE_FORCES, h->d_out);
+        if (e == cudaSuccess)
+          e = launch_min_iteration(h->args, h->d_out, scratch, step_dt, dmax, ftol, h->f64, b, h->stream);
+      }
+      launched += k;
+      if (e == cudaSuccess) e = cudaMemcpyAsync(hs.data(), scratch, hs.size(), cudaMemcpyDeviceToHost, h->stream);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+      if (e != cudaSuccess) break;
+      min_progress(hs.data(), &done, &fn, &conv);
+      if (conv) break;
+    }
+    if (e == cudaSuccess && !conv) {
+      // |F| at the final positions (the force kernel of one more iteration; it moves
+      // nothing when converged, and otherwise the count of moves is already max_iters)
       if (!(h->p.flags & IONTRAP_COULOMB_OFF)) e = launch_mode(h, MODE_FORCES, h->d_out);
       if (e == cudaSuccess)
-        e = launch_min_iteration(h->args, h->d_out, scratch, step_dt, dmax, ftol, h->f64, b, h->stream);
+        e = launch_min_iteration(h->args, h->d_out, scratch, step_dt, dmax, std::numeric_limits<double>::infinity(),
+                                 h->f64, b, h->stream);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(hs.data(), scratch, hs.size(), cudaMemcpyDeviceToHost, h->stream);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+      if (e == cudaSuccess) {
+        long long d2;
+        int c2;
+        min_progress(hs.data(), &d2, &fn, &c2);
+      }
     }
-    launched += k;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(hs.data(), scratch, hs.size(), cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) break;
-    min_progress(hs.data(), &done, &fn, &conv);
-    if (conv) break;
+    cudaFree(scratch);
+    if (e != cudaSuccess) return cuda_status(h, e);
   }
-  if (e == cudaSuccess && !conv) {
-    // |F| at the final positions (the force kernel of one more iteration; it moves
-    // nothing when converged, and otherwise the count of moves is already max_iters)
-    if (!(h->p.flags & IONTRAP_COULOMB_OFF)) e = launch_mode(h, MODE_FORCES, h->d_out);
-    if (e == cudaSuccess)
-      e = launch_min_iteration(h->args, h->d_out, scratch, step_dt, dmax, std::numeric_limits<double>::infinity(),
-                               h->f64, b, h->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(hs.data(), scratch, hs.size(), cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    if (e == cudaSuccess) {
-      long long d2;
-      int c2;
-      min_progress(hs.data(), &d2, &fn, &c2);
-    }
-  }
-  cudaFree(scratch);
-  if (e != cudaSuccess) return cuda_status(h, e);
   if (iters) *iters = done;
   if (fnorm) *fnorm = fn;
   // the minimum at rest: v = 0, a_n evaluated under the handle's forces

@@ -109,6 +109,13 @@ struct F64View {
   int I, rows, cols, warps;
 };
 
+// Result of a minimisation launch (minimize.cu).
+struct MinResult {
+  long long iters;  // moves made so far
+  double fnorm;     // |F| of the last force evaluation
+  int converged;
+};
+
 // ------------------------------------------------------------------ PTX helpers
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -170,9 +177,74 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s
 
+// ------------------------------------------------------------------ grid-wide counters
+__device__ __forceinline__ unsigned ld_relaxed_u32(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
+// Wait of a persistent form's poller until *ctr >= target: the counter alone is polled,
+// the timeout flag and the clock every 64 polls.  ACQ: acquire loads (no fence needed
+// after a successful wait).  Gives up (false) after limit ns, setting the timeout flag,
+// or when another CTA has set it.
+template <bool ACQ>
+static __device__ __noinline__ bool poll_wait(const unsigned* ctr, unsigned target, int* err, unsigned long long limit) {
+  const unsigned long long t0 = globaltimer_ns();
+  for (unsigned it = 1;; ++it) {
+    unsigned c;
+    if (ACQ)
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(ctr) : "memory");
+    else
+      c = ld_relaxed_u32(ctr);
+    if (c >= target) return true;
+    if ((it & 63) == 0) {
+      if (*(volatile int*)err & ERR_TIMEOUT) return false;
+      if (globaltimer_ns() - t0 > limit) {
+        atomicOr(err, ERR_TIMEOUT);
+        return false;
+      }
+    }
+  }
+}
+
+// A CTA's arrival on a counter: release at GPU scope orders the CTA's earlier writes
+// (after a CTA barrier) before the increment.
+__device__ __forceinline__ void arrive_release(unsigned* ctr) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr) : "memory");
+}
+
 // Phase timestamp of this CTA into the optional trace buffer (thread 0 only).
 __device__ __forceinline__ void trace_mark(unsigned long long* trace, long long slot) {
   if (trace && threadIdx.x == 0) trace[slot] = globaltimer_ns();
+}
+
+// ------------------------------------------------------------------ float <-> double
+// (double)x without the FP64-rate conversion: normal floats and zeros by their bits.
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  if (m - 0x00800000u < 0x7f000000u)  // normal
+    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+  if (m == 0u) return __hiloint2double((int)b, 0);
+  return (double)x;
+}
+
+// hi = fl(x), lo = fl(x - hi) without FP64-rate operations: the mantissa's top 24 bits
+// rounded to nearest even, the signed remainder converted and scaled (exact but for its own
+// rounding).  Exponents outside the range where hi and lo are both normal take the plain way.
+__device__ __forceinline__ void split_hilo(double x, float& hi, float& lo) {
+  const unsigned xh = (unsigned)__double2hiint(x), xl = (unsigned)__double2loint(x);
+  const unsigned e = (xh >> 20) & 0x7ffu;
+  if (e - 960u <= 180u) {
+    const unsigned m = ((xh & 0xfffffu) << 3) | (xl >> 29), rem = xl & 0x1fffffffu;
+    const unsigned up = (rem + (m & 1u) > 0x10000000u) ? 1u : 0u;
+    hi = __uint_as_float((xh & 0x80000000u) | (((e - 896u) << 23) + m + up));
+    const int r = (int)rem - (int)(up << 29);
+    lo = __int2float_rn((xh >> 31) ? -r : r) * __uint_as_float((e - 948u) << 23);
+    return;
+  }
+  hi = __double2float_rn(x);
+  lo = __double2float_rn(x - (double)hi);
 }
 
 // ------------------------------------------------------------------ FP32 pair terms
@@ -324,6 +396,37 @@ __device__ __forceinline__ void rp_chunk_i2(const float* __restrict__ sj, const 
   }
 }
 
+// The cluster kernels keep positions as records of four ions: rows x, y, z hi and x, y, z lo of
+// four floats (96 bytes), so one address and constant offsets reach all of a record.  Float of
+// ion e, row r:
+constexpr int kRpcRec = 24;
+__device__ __forceinline__ int rpc_at(int e, int r) { return (e >> 2) * kRpcRec + 4 * r + (e & 3); }
+
+// Part [j0, j0 + JP) (one chunk) of ion i's sum: the bits rp_chunk and the Kahan sum of one
+// chunk give.  Every part tests for the self pair: one copy of the loop in the instruction
+// cache is worth more than its two selects.
+template <bool UNITW>
+__device__ __forceinline__ void rec_part(const float* sb, const float* wz, int j0, int JP, int i, const float2 (&nh)[3],
+                                         const float2 (&nl)[3], float (&out)[3]) {
+  float2 acc[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  const float4* rec = reinterpret_cast<const float4*>(sb + rpc_at(j0, 0));
+  const float4* sw = reinterpret_cast<const float4*>(wz + j0);
+#pragma unroll 2
+  for (int q = 0; q < JP; q += 4, rec += kRpcRec / 4) {
+    const float4 hx = rec[0], hy = rec[1], hz = rec[2], lx = rec[3], ly = rec[4], lz = rec[5];
+    float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (!UNITW) w = sw[q >> 2];
+    rp_pair2<true, UNITW>(make_float2(hx.x, hx.y), make_float2(hy.x, hy.y), make_float2(hz.x, hz.y),
+                          make_float2(lx.x, lx.y), make_float2(ly.x, ly.y), make_float2(lz.x, lz.y),
+                          make_float2(w.x, w.y), j0 + q, i, nh, nl, acc);
+    rp_pair2<true, UNITW>(make_float2(hx.z, hx.w), make_float2(hy.z, hy.w), make_float2(hz.z, hz.w),
+                          make_float2(lx.z, lx.w), make_float2(ly.z, ly.w), make_float2(lz.z, lz.w),
+                          make_float2(w.z, w.w), j0 + q + 2, i, nh, nl, acc);
+  }
+#pragma unroll
+  for (int d = 0; d < 3; ++d) out[d] = 0.0f + (acc[d].x + acc[d].y);
+}
+
 // ------------------------------------------------------------------ split partials
 // RF phase at the force time of a launch in the given mode.
 __device__ __forceinline__ double force_time_cos(const StepArgs& A, long long ns) {
@@ -433,6 +536,11 @@ __device__ __forceinline__ void normals3_f64(unsigned long long seed, long long 
 // operations, hence the same bits.
 __device__ __forceinline__ double half_kick(double v, double a, double hdt) { return __fma_rn(hdt, a, v); }
 __device__ __forceinline__ double drift(double x, double vh, double dt) { return __fma_rn(dt, vh, x); }
+
+// Sum of three squares, in the rounding order both minimisers use.
+__device__ __forceinline__ double square3(double a, double b, double c) {
+  return __fma_rn(c, c, __fma_rn(a, a, __dmul_rn(b, b)));
+}
 
 // Entry i of pair stream b for the next positions xn (FP64 form: double4_32a; FP32 form:
 // hi = fl(xn), lo = fl(xn - hi)).

@@ -102,15 +102,16 @@ __global__ void __launch_bounds__(kMinThreads) k_min_force(const __grid_constant
     const SpeciesDev& sd = A.spc[A.sp[i]];
     double k[3];
     trap_springs(A.trap, sd, 0.0, k);
+    double F[3], v[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const double x = A.x[c * n + i];
-      const double a = A.coul[c * n + i] + (-k[c] * x);
-      const double F = sd.mass * a;
+      const double a = __fma_rn(-k[c], A.x[c * n + i], A.coul[c * n + i]);
+      F[c] = sd.mass * a;
+      v[c] = A.v[c * n + i];
       A.a[c * n + i] = a;
-      acc2[0] += F * F;
-      acc2[1] += A.v[c * n + i] * F;
     }
+    acc2[0] += square3(F[0], F[1], F[2]);
+    acc2[1] += __fma_rn(v[2], F[2], __fma_rn(v[1], F[1], __dmul_rn(v[0], F[0])));
   }
   block_reduce2<0>(acc2, sh);
   if (threadIdx.x == 0) {
@@ -144,16 +145,15 @@ __global__ void __launch_bounds__(kMinThreads) k_min_kick(const __grid_constant_
   for (long long i = blockIdx.x * (long long)kMinThreads + threadIdx.x; i < n;
        i += (long long)gridDim.x * kMinThreads) {
     const SpeciesDev& sd = A.spc[A.sp[i]];
-    double d2 = 0.0;
+    double d[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const double a = A.a[c * n + i];
-      const double v = scale * (sd.mass * a) + A.dt * a;
+      const double v = __fma_rn(scale, __dmul_rn(sd.mass, a), __dmul_rn(A.dt, a));
       A.v[c * n + i] = v;
-      const double d = A.dt * v;
-      d2 += d * d;
+      d[c] = A.dt * v;
     }
-    dm[0] = fmax(dm[0], sqrt(d2));
+    dm[0] = fmax(dm[0], sqrt(square3(d[0], d[1], d[2])));
   }
   block_reduce2<1>(dm, sh);
   if (threadIdx.x == 0) A.part[2 * blockIdx.x] = dm[0];
@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(kMinThreads) k_min_move(const __grid_constant_
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const double v = A.v[c * n + i];
-      xn[c] = A.x[c * n + i] + s * (A.dt * v);
+      xn[c] = __fma_rn(s, A.dt * v, A.x[c * n + i]);
       A.x[c * n + i] = xn[c];
       A.v[c * n + i] = s * v;
     }

@@ -32,42 +32,6 @@ struct GpArgs {
   int Lmax;        // entries per stream of the largest segment (shared-memory extent)
 };
 
-__device__ __forceinline__ unsigned ld_relaxed_u32(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
-// Wait of a persistent form's poller until *ctr >= target: the counter alone is polled,
-// the timeout flag and the clock every 64 polls.  ACQ: acquire loads (no fence needed
-// after a successful wait).  Gives up (false) after limit ns, setting the timeout flag,
-// or when another CTA has set it.
-template <bool ACQ>
-__device__ __noinline__ bool poll_wait(const unsigned* ctr, unsigned target, int* err, unsigned long long limit) {
-  const unsigned long long t0 = globaltimer_ns();
-  for (unsigned it = 1;; ++it) {
-    unsigned c;
-    if (ACQ)
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(ctr) : "memory");
-    else
-      c = ld_relaxed_u32(ctr);
-    if (c >= target) return true;
-    if ((it & 63) == 0) {
-      if (*(volatile int*)err & ERR_TIMEOUT) return false;
-      if (globaltimer_ns() - t0 > limit) {
-        atomicOr(err, ERR_TIMEOUT);
-        return false;
-      }
-    }
-  }
-}
-
-// A CTA's arrival on a counter: release at GPU scope orders the CTA's earlier writes
-// (after a CTA barrier) before the increment.
-__device__ __forceinline__ void arrive_release(unsigned* ctr) {
-  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr) : "memory");
-}
-
 template <int W>
 __global__ void __launch_bounds__(32 * W, 16 / W) k_step_f32_gp(const __grid_constant__ StepArgs A, const GpArgs P) {
   constexpr int T = 32 * W;
