@@ -376,8 +376,6 @@ void default_config(int64_t n, int f64, int sms, int* T, int* I, int* packed, in
     *packed = 0;
   } else if (n <= 8192) {
     *T = 64, *I = 1, *packed = 0;
-  } else if (n <= 32768) {
-    *T = 128, *I = 4, *packed = 1;
   } else {
     *T = 128, *I = 4, *packed = 1;
   }
@@ -408,6 +406,11 @@ void default_config(int64_t n, int f64, int sms, int* T, int* I, int* packed, in
   if (f64) js = std::min<int64_t>(js, kMaxJsplitF64);
   if (!*fused && cdiv(n, js) > kMaxSplitsUnfused) js = cdiv(n, kMaxSplitsUnfused);
   *jsplit = (int)js;
+  // above 8192: j-ranges laid out for blocks of 512 ions, summed by CTAs of 64 threads and 2
+  // ions each (the same bits: they depend on the j-ranges only).  Eight times the CTAs, and
+  // the last of an i-block integrates 128 ions instead of 512 (us per step, 128 x 4 against
+  // 64 x 2: n = 9001: 84 -> 64, 16384: 183 -> 153, 32768: 654 -> 564)
+  if (!f64 && n > 8192) *T = 64, *I = 2;
   // 2048 < n <= 8192: the cluster + warp-split form (4 warps, 2 ions per lane, 8-CTA
   // clusters) measured fastest (20.8 us/step at n = 4096 against 24.7 for the others)
   if (!f64 && n > 2048 && n <= 8192) {
