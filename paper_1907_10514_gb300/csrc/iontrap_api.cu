@@ -8,6 +8,7 @@
 // for the remainder; no host round trip happens between steps.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -110,7 +111,9 @@ struct iontrap {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   cudaStream_t cap = nullptr;  // private stream used only to capture the step graph
-  // device buffers
+  // device buffers; one block holds a header (step, error flags, completed i-blocks), x, v, a
+  // and the species indices, so that a state travels in one copy
+  char* d_block = nullptr;
   double *d_x = nullptr, *d_v = nullptr, *d_a = nullptr, *d_out = nullptr;
   unsigned char* d_sp = nullptr;
   void* d_pair[2] = {nullptr, nullptr};
@@ -575,6 +578,89 @@ void dev_free(const iontrap* h, void* p) {
   if (p) cudaFreeAsync(p, h->stream);
 }
 
+// What a handle's block begins with.
+struct Header {
+  long long step;
+  int err;
+  unsigned done;
+};
+constexpr size_t kHeaderBytes = 64;
+
+// Pinned host memory for the copies of small states: a driver call and a wait cost ~10 us each
+// on GB300, the copy of a few hundred KB through pinned memory less.  Buffers are kept for the
+// next call, at most kStagingKeep of them, none above kStagingMax bytes; p is null where the
+// copy is larger (or none can be had) and goes straight to and from the caller's arrays.
+constexpr size_t kStagingMax = 256 * 1024;
+constexpr size_t kStagingKeep = 16;
+std::mutex g_staging_mu;
+std::vector<char*> g_staging;
+
+struct Staging {
+  char* p = nullptr;
+  explicit Staging(size_t bytes) {
+    if (bytes > kStagingMax) return;
+    {
+      std::lock_guard<std::mutex> lock(g_staging_mu);
+      if (!g_staging.empty()) {
+        p = g_staging.back();
+        g_staging.pop_back();
+      }
+    }
+    if (p) return;
+    void* q = nullptr;
+    if (cudaHostAlloc(&q, kStagingMax, cudaHostAllocPortable) == cudaSuccess)
+      p = static_cast<char*>(q);
+    else
+      cudaGetLastError();
+  }
+  ~Staging() {
+    if (!p) return;
+    {
+      std::lock_guard<std::mutex> lock(g_staging_mu);
+      if (g_staging.size() < kStagingKeep) {
+        g_staging.push_back(p);
+        return;
+      }
+    }
+    cudaFreeHost(p);
+  }
+  Staging(const Staging&) = delete;
+  Staging& operator=(const Staging&) = delete;
+};
+
+// Wait for the handle's stream, take over its error flags, and copy out what is wanted of the
+// state (null: not).  After a non-finite or timed-out step the state is copied all the same;
+// other failures copy nothing.  *dstep: the device's step index.
+int fetch(iontrap* h, double* x, double* v, double* a, long long* dstep) {
+  const size_t vec = 3 * (size_t)h->n * sizeof(double);
+  const size_t want = a ? 3 * vec : (v ? 2 * vec : (x ? vec : 0));
+  Staging stage(kHeaderBytes + want);
+  cudaError_t e = cudaSuccess;
+  Header head{};
+  if (stage.p) {
+    e = cudaMemcpyAsync(stage.p, h->d_block, kHeaderBytes + want, cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e == cudaSuccess) std::memcpy(&head, stage.p, sizeof(head));
+  } else {
+    e = cudaStreamSynchronize(h->stream);
+    if (e == cudaSuccess) e = cudaMemcpy(&head, h->d_block, sizeof(head), cudaMemcpyDeviceToHost);
+  }
+  if (e != cudaSuccess) return cuda_status(h, e);
+  if (head.err & ERR_TIMEOUT) set_status(h, IONTRAP_ETIMEOUT);
+  if (head.err & ERR_NONFINITE) set_status(h, IONTRAP_ENONFINITE);
+  if (dstep) *dstep = head.step;
+  if (h->status != IONTRAP_OK && h->status != IONTRAP_ENONFINITE && h->status != IONTRAP_ETIMEOUT) return h->status;
+  double* const out[3] = {x, v, a};
+  for (int k = 0; k < 3 && e == cudaSuccess; ++k)
+    if (out[k]) {
+      if (stage.p)
+        std::memcpy(out[k], stage.p + kHeaderBytes + k * vec, vec);
+      else
+        e = cudaMemcpy(out[k], h->d_x + 3 * (size_t)k * h->n, vec, cudaMemcpyDeviceToHost);
+    }
+  return e == cudaSuccess ? h->status : cuda_status(h, e);
+}
+
 // (Re)allocate the scratch that depends on the tile configuration.
 int alloc_scratch(iontrap* h) {
   const int64_t splits = splits_of(h);
@@ -742,8 +828,7 @@ int reevaluate(iontrap* h) {
 
 void free_all(iontrap* h) {
   destroy_graph(h);
-  void* ptrs[] = {h->d_x, h->d_v, h->d_a, h->d_out, h->d_sp, h->d_pair[0], h->d_pair[1],
-                  h->d_part, h->d_cnt, h->d_done, h->d_step, h->d_err, h->d_gsync, h->d_snap};
+  void* ptrs[] = {h->d_block, h->d_out, h->d_pair[0], h->d_pair[1], h->d_part, h->d_cnt, h->d_gsync, h->d_snap};
   for (void* q : ptrs) dev_free(h, q);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   if (h->cap) cudaStreamDestroy(h->cap);
@@ -914,12 +999,8 @@ int iontrap_create(const iontrap_species* species, int n_species, const uint8_t*
 
   const size_t vec = 3 * (size_t)n * sizeof(double);
   const size_t pair = (size_t)n * (h->f64 ? sizeof(double4_32a) : 2 * sizeof(float4));
-  bool ok = dev_alloc(h, &h->d_x, vec) == cudaSuccess && dev_alloc(h, &h->d_v, vec) == cudaSuccess &&
-            dev_alloc(h, &h->d_a, vec) == cudaSuccess && dev_alloc(h, &h->d_sp, (size_t)n) == cudaSuccess &&
-            dev_alloc(h, &h->d_pair[0], pair) == cudaSuccess && dev_alloc(h, &h->d_pair[1], pair) == cudaSuccess &&
-            dev_alloc(h, &h->d_done, sizeof(unsigned)) == cudaSuccess &&
-            dev_alloc(h, &h->d_step, sizeof(long long)) == cudaSuccess &&
-            dev_alloc(h, &h->d_err, sizeof(int)) == cudaSuccess;
+  const bool ok = dev_alloc(h, &h->d_block, kHeaderBytes + 3 * vec + (size_t)n) == cudaSuccess &&
+                  dev_alloc(h, &h->d_pair[0], pair) == cudaSuccess && dev_alloc(h, &h->d_pair[1], pair) == cudaSuccess;
   if (!ok) {
     free_all(h);
     delete h;
@@ -935,6 +1016,13 @@ int iontrap_create(const iontrap_species* species, int n_species, const uint8_t*
       A.p64[b] = nullptr;
     }
   }
+  h->d_step = reinterpret_cast<long long*>(h->d_block + offsetof(Header, step));
+  h->d_err = reinterpret_cast<int*>(h->d_block + offsetof(Header, err));
+  h->d_done = reinterpret_cast<unsigned*>(h->d_block + offsetof(Header, done));
+  h->d_x = reinterpret_cast<double*>(h->d_block + kHeaderBytes);
+  h->d_v = h->d_x + 3 * n;
+  h->d_a = h->d_v + 3 * n;
+  h->d_sp = reinterpret_cast<unsigned char*>(h->d_a + 3 * n);
   A.x = h->d_x;
   A.v = h->d_v;
   A.a = h->d_a;
@@ -948,21 +1036,33 @@ int iontrap_create(const iontrap_species* species, int n_species, const uint8_t*
     delete h;
     return st;
   }
-  long long s0 = step0;
   cudaError_t e = cudaSuccess;
   auto chk = [&](cudaError_t r) {
     if (e == cudaSuccess) e = r;
   };
-  chk(cudaMemcpyAsync(h->d_x, x0, vec, cudaMemcpyHostToDevice, h->stream));
-  if (v0)
-    chk(cudaMemcpyAsync(h->d_v, v0, vec, cudaMemcpyHostToDevice, h->stream));
-  else
-    chk(cudaMemsetAsync(h->d_v, 0, vec, h->stream));
-  chk(cudaMemcpyAsync(h->d_sp, species_of_ion, (size_t)n, cudaMemcpyHostToDevice, h->stream));
-  chk(cudaMemcpyAsync(h->d_step, &s0, sizeof(s0), cudaMemcpyHostToDevice, h->stream));
-  chk(cudaMemsetAsync(h->d_done, 0, sizeof(unsigned), h->stream));
-  chk(cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream));
-  chk(cudaMemsetAsync(h->d_a, 0, vec, h->stream));
+  const Header head{step0, 0, 0u};
+  Staging stage(kHeaderBytes + 3 * vec + (size_t)n);
+  if (char* s = stage.p) {
+    std::memset(s, 0, kHeaderBytes);
+    std::memcpy(s, &head, sizeof(head));
+    std::memcpy(s + kHeaderBytes, x0, vec);
+    if (v0)
+      std::memcpy(s + kHeaderBytes + vec, v0, vec);
+    else
+      std::memset(s + kHeaderBytes + vec, 0, vec);
+    std::memset(s + kHeaderBytes + 2 * vec, 0, vec);
+    std::memcpy(s + kHeaderBytes + 3 * vec, species_of_ion, (size_t)n);
+    chk(cudaMemcpyAsync(h->d_block, s, kHeaderBytes + 3 * vec + (size_t)n, cudaMemcpyHostToDevice, h->stream));
+  } else {
+    chk(cudaMemcpyAsync(h->d_x, x0, vec, cudaMemcpyHostToDevice, h->stream));
+    if (v0)
+      chk(cudaMemcpyAsync(h->d_v, v0, vec, cudaMemcpyHostToDevice, h->stream));
+    else
+      chk(cudaMemsetAsync(h->d_v, 0, vec, h->stream));
+    chk(cudaMemcpyAsync(h->d_sp, species_of_ion, (size_t)n, cudaMemcpyHostToDevice, h->stream));
+    chk(cudaMemcpyAsync(h->d_block, &head, sizeof(head), cudaMemcpyHostToDevice, h->stream));
+    chk(cudaMemsetAsync(h->d_a, 0, vec, h->stream));
+  }
   chk(launch_prep(h, (int)(step0 & 1)));
   chk(launch_mode(h, MODE_INIT, nullptr));
   chk(cudaStreamSynchronize(h->stream));
@@ -1222,33 +1322,32 @@ int iontrap_step_record(iontrap_t* h, int64_t n_steps, int64_t every, uint32_t f
 int iontrap_sync(iontrap_t* h) {
   if (!h) return IONTRAP_EINVAL;
   DeviceGuard g(h->device);
-  cudaError_t e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return cuda_status(h, e);
-  int err = 0;
-  e = cudaMemcpy(&err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_status(h, e);
-  if (err & ERR_TIMEOUT) set_status(h, IONTRAP_ETIMEOUT);
-  if (err & ERR_NONFINITE) set_status(h, IONTRAP_ENONFINITE);
-  return h->status;
+  return fetch(h, nullptr, nullptr, nullptr, nullptr);
 }
 
-int iontrap_state(iontrap_t* h, double* x, double* v, int64_t* step, double* t) {
-  if (!h) return IONTRAP_EINVAL;
-  const int st = iontrap_sync(h);
-  if (st != IONTRAP_OK && st != IONTRAP_ENONFINITE && st != IONTRAP_ETIMEOUT) return st;
+}  // extern "C"
+
+namespace {
+
+// iontrap_state and iontrap_checkpoint: the step index is compared with the enqueued one.
+int read_state(iontrap* h, double* x, double* v, double* a, int64_t* step, double* t) {
   DeviceGuard g(h->device);
-  const size_t vec = 3 * (size_t)h->n * sizeof(double);
-  cudaError_t e = cudaSuccess;
-  if (x) e = cudaMemcpy(x, h->d_x, vec, cudaMemcpyDeviceToHost);
-  if (v && e == cudaSuccess) e = cudaMemcpy(v, h->d_v, vec, cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_status(h, e);
-  long long dstep = 0;
-  e = cudaMemcpy(&dstep, h->d_step, sizeof(dstep), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_status(h, e);
+  long long dstep = -1;
+  const int st = fetch(h, x, v, a, &dstep);
+  if (st != IONTRAP_OK && st != IONTRAP_ENONFINITE && st != IONTRAP_ETIMEOUT) return st;
   if (dstep != h->step && h->status == IONTRAP_OK) set_status(h, IONTRAP_ETIMEOUT);
   if (step) *step = dstep;
   if (t) *t = (double)dstep * h->p.dt;
   return h->status;
+}
+
+}  // namespace
+
+extern "C" {
+
+int iontrap_state(iontrap_t* h, double* x, double* v, int64_t* step, double* t) {
+  if (!h) return IONTRAP_EINVAL;
+  return read_state(h, x, v, nullptr, step, t);
 }
 
 int iontrap_forces(iontrap_t* h, double* acc) {
@@ -1273,14 +1372,7 @@ int iontrap_forces(iontrap_t* h, double* acc) {
 
 int iontrap_checkpoint(iontrap_t* h, double* x, double* v, double* a, int64_t* step) {
   if (!h) return IONTRAP_EINVAL;
-  int st = iontrap_state(h, x, v, step, nullptr);
-  if (st) return st;
-  DeviceGuard g(h->device);
-  if (a) {
-    cudaError_t e = cudaMemcpy(a, h->d_a, 3 * (size_t)h->n * sizeof(double), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_status(h, e);
-  }
-  return h->status;
+  return read_state(h, x, v, a, step, nullptr);
 }
 
 int iontrap_restore(iontrap_t* h, const double* x, const double* v, const double* a, int64_t step) {
@@ -1291,13 +1383,25 @@ int iontrap_restore(iontrap_t* h, const double* x, const double* v, const double
   if (st) return st;
   DeviceGuard g(h->device);
   const size_t vec = 3 * (size_t)h->n * sizeof(double);
-  long long s = step;
-  cudaError_t e = cudaMemcpyAsync(h->d_x, x, vec, cudaMemcpyHostToDevice, h->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_v, v, vec, cudaMemcpyHostToDevice, h->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_a, a, vec, cudaMemcpyHostToDevice, h->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_step, &s, sizeof(s), cudaMemcpyHostToDevice, h->stream);
+  const Header head{step, 0, 0u};  // the flags and the counter are clear after a sync without errors
+  cudaError_t e = cudaSuccess;
+  Staging stage(kHeaderBytes + 3 * vec);
+  if (char* p = stage.p) {
+    std::memset(p, 0, kHeaderBytes);
+    std::memcpy(p, &head, sizeof(head));
+    std::memcpy(p + kHeaderBytes, x, vec);
+    std::memcpy(p + kHeaderBytes + vec, v, vec);
+    std::memcpy(p + kHeaderBytes + 2 * vec, a, vec);
+    e = cudaMemcpyAsync(h->d_block, p, kHeaderBytes + 3 * vec, cudaMemcpyHostToDevice, h->stream);
+  } else {
+    e = cudaMemcpyAsync(h->d_x, x, vec, cudaMemcpyHostToDevice, h->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_v, v, vec, cudaMemcpyHostToDevice, h->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_a, a, vec, cudaMemcpyHostToDevice, h->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_block, &head, sizeof(head), cudaMemcpyHostToDevice, h->stream);
+  }
   if (e == cudaSuccess) e = launch_restore(h, (int)((step + 1) & 1));
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  const cudaError_t es = cudaStreamSynchronize(h->stream);  // also before the staging goes back
+  if (e == cudaSuccess) e = es;
   if (e != cudaSuccess) return cuda_status(h, e);
   h->step = step;
   return h->status;
