@@ -1,83 +1,155 @@
 // forces_noalloc.cu -- Coulomb accelerations without any device allocation.
 //
 // iontrap_forces evaluates the force kernel on a handle, and a handle owns device
-// buffers that iontrap_create obtained with cudaMalloc.  Some callers cannot allocate:
-// a process that hands all of its device memory to its own pool up front and forbids
-// allocations behind its back, a host application that loads this library as a plugin
-// and owns every device buffer itself, or a latency-critical loop that must not pay
-// for cudaMalloc's implicit synchronisation.  For them, iontrap_forces_noalloc takes
-// the positions and the output in the caller's device memory and keeps every piece of
-// scratch the force kernel needs -- the FP32 hi/lo pair stream, the per-split partial
-// sums and the arrival counters -- in one fixed array of device memory that is part of
-// the library image itself (g_scratch below).  Every GPU that loads the library holds
-// that array until the process exits.
+// buffers.  Some callers cannot allocate: a process that hands all of its device memory
+// to its own pool up front and forbids allocations behind its back, a host application
+// that loads this library as a plugin and owns every device buffer itself, or a
+// latency-critical loop that must not pay for cudaMalloc's implicit synchronisation.  For
+// them, iontrap_forces_noalloc takes the positions and the output in the caller's device
+// memory and needs nothing else: one kernel, whose partial sums never leave the chip.
 //
-// Limits and sharing: at most kNoAllocMaxIons ions per call (larger calls return
-// IONTRAP_ETOOLARGE without launching anything).  All calls on a device share the
-// one array, which keeps whatever the previous call left in it; each call clears the
-// counters it relies on before it launches.  Two calls whose work overlaps on the GPU
-// (different streams, or different host threads) race on the array and give wrong
-// results: serialise them.
+// A cluster of S <= 8 CTAs sums 32 or 64 ions (one per lane, or two packed), CTA s against the
+// s-th of S equal j-ranges.  Warp w of a CTA takes the range's w-th chunk of 128 j: it splits the
+// FP64 positions into hi/lo floats itself (integer operations: the FP64 pipe would take
+// longer than the pairs at small n), and its plain FP32 chunk sums are Kahan-added in chunk
+// order by the CTA, the CTAs' (sum, compensation) pairs merged in range order through
+// distributed shared memory.  That is the summation order (and the bits) of the last-CTA step
+// form with these j-ranges, without its scratch, counters and clears.
+//
+// Bound by the FP32 pipe at n = 8192 (half of its rate: few warps, the split of the positions
+// in every CTA) and by the launch and one chunk's latency below ~2000.  Measured back to back on
+// GB300, us per call, the previous two clears and two launches against this kernel: n = 64:
+// 17 -> 8.3, 1000: 21 -> 10.3, 3000: 32 -> 16.3, 5000: 46 -> 27, 8192: 77 -> 55.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
-#include <mutex>
 
 #include "iontrap_internal.cuh"
 
-namespace it {
-const void* step_kernel(int T, int I, int packed, int fused);
-const void* prep_kernel();
-}  // namespace it
-
+namespace cg = cooperative_groups;
 using namespace it;
 
 namespace {
 
 constexpr long long kNoAllocMaxIons = 8192;
 constexpr int kNoAllocMaxSplits = 8;
-constexpr int kNoAllocThreads = 64;  // force kernel: 64 threads, one ion per thread
+constexpr int kMaxChunks = (int)(kNoAllocMaxIons / kNoAllocMaxSplits / kSeg);  // warps per CTA: 8
 
-// Byte layout of the scratch array.
-constexpr size_t kOffStep = 0;     // long long, kept 0 (pair stream buffer 0 is used)
-constexpr size_t kOffErr = 8;      // int error flags
-constexpr size_t kOffDone = 12;    // unsigned, completed i-blocks
-constexpr size_t kOffCnt = 256;    // unsigned[i-blocks], per-i-block arrival counters
-constexpr size_t kCntBytes = ((kNoAllocMaxIons / kNoAllocThreads) * sizeof(unsigned) + 255) / 256 * 256;
-constexpr size_t kOffPair = kOffCnt + kCntBytes;  // float4 hi[n], lo[n]
-constexpr size_t kPairBytes = (size_t)kNoAllocMaxIons * 2 * sizeof(float4);
-constexpr size_t kOffPart = kOffPair + kPairBytes;  // 32-byte records, split * n + i
-constexpr size_t kPartBytes = (size_t)kNoAllocMaxSplits * kNoAllocMaxIons * 32;
-constexpr size_t kScratchBytes = kOffPart + kPartBytes;  // 2.25 MiB + 768 B
+struct ForcesArgs {
+  int n, jsplit;
+  const unsigned char* sp;
+  const double* x;
+  double* out;
+  double coul[IONTRAP_MAX_SPECIES];
+  float w[IONTRAP_MAX_SPECIES];
+};
 
-static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
-
-// Device address of g_scratch per device.  In host code the name g_scratch is only a
-// host-side stand-in for the symbol, so the address is looked up with that device
-// current by cudaGetSymbolAddress.  The lookup is repeated on every call made outside
-// stream capture, because the address belongs to the device's current context: after a
-// cudaDeviceReset (or any other teardown of the primary context) the module is loaded
-// again and the array may sit elsewhere.  A call made while its stream is being captured
-// uses the address the last uncaptured call on that device found.
-std::mutex g_mu;
-constexpr int kMaxDevices = 64;
-unsigned char* g_addr[kMaxDevices] = {};
-
-int scratch_for_device(int dev, cudaStream_t stream, unsigned char** out) {
-  if (dev < 0 || dev >= kMaxDevices) return IONTRAP_ECUDA;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(stream, &cs) != cudaSuccess) return IONTRAP_ECUDA;
-  std::lock_guard<std::mutex> lock(g_mu);
-  if (cs == cudaStreamCaptureStatusNone) {
-    void* p = nullptr;
-    const cudaError_t e = cudaGetSymbolAddress(&p, g_scratch);
-    if (e != cudaSuccess || !p) return IONTRAP_ECUDA;
-    g_addr[dev] = static_cast<unsigned char*>(p);
+// I ions per lane: 1, or 2 packed.
+template <int I, bool UNITW>
+__global__ void __launch_bounds__(32 * kMaxChunks) k_forces_cluster(const __grid_constant__ ForcesArgs A) {
+  constexpr int kBlockIons = 32 * I;
+  __shared__ __align__(16) float4 sh[kMaxChunks][kSeg], sl[kMaxChunks][kSeg];
+  __shared__ float s_sum[kMaxChunks][3][kBlockIons];   // chunk sums; row 0 then the CTA's Kahan sum
+  __shared__ float s_comp[3][kBlockIons];              // and compensation
+  cg::cluster_group cluster = cg::this_cluster();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, threads = blockDim.x;
+  const int n = A.n, i0 = blockIdx.x * kBlockIons;
+  const int j0 = blockIdx.y * A.jsplit, j1 = min(n, j0 + A.jsplit);
+  const int chunks = (j1 - j0 + kSeg - 1) / kSeg;
+  const int jc = j0 + warp * kSeg, jn = min(kSeg, j1 - jc);
+  if (jn > 0) {
+    // every load first (one trip to memory), then the conversions
+    constexpr int Q = kSeg / 32;
+    double x[Q + I][3];
+    float w[Q];
+    long long ii[I];
+#pragma unroll
+    for (int q = 0; q < Q + I; ++q) {
+      const int e = q < Q ? jc + 32 * q + lane : i0 + 32 * (q - Q) + lane;
+      const bool on = q < Q ? 32 * q + lane < jn : e < n;
+      if (q >= Q) ii[q - Q] = e;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) x[q][d] = on ? A.x[d * n + e] : 1.0;  // (unused)
+      if (q < Q) w[q] = UNITW ? 1.0f : (on ? A.w[A.sp[e]] : 0.0f);
+    }
+    float2 nxh[1][3], nxl[1][3], acc[1][3];
+#pragma unroll
+    for (int q = 0; q < Q + I; ++q) {
+      float h[3], l[3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) split_hilo(x[q][d], h[d], l[d]);
+      if (q < Q) {
+        sh[warp][32 * q + lane] = make_float4(h[0], h[1], h[2], w[q]);
+        sl[warp][32 * q + lane] = make_float4(l[0], l[1], l[2], 0.0f);
+      } else {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          if (q == Q)
+            nxh[0][d].x = -h[d], nxl[0][d].x = -l[d];
+          else
+            nxh[0][d].y = -h[d], nxl[0][d].y = -l[d];
+          acc[0][d] = make_float2(0.f, 0.f);
+        }
+      }
+    }
+    __syncwarp();
+    const bool diag = jc < i0 + kBlockIons && i0 < jc + jn;
+    if constexpr (I == 1) {
+      const float h1[1][3] = {{nxh[0][0].x, nxh[0][1].x, nxh[0][2].x}};
+      const float l1[1][3] = {{nxl[0][0].x, nxl[0][1].x, nxl[0][2].x}};
+      float a1[1][3] = {{0.f, 0.f, 0.f}};
+      if (diag)
+        segment_f32<1, true, UNITW>(sh[warp], sl[warp], jn, jc, h1, l1, ii, a1);
+      else
+        segment_f32<1, false, UNITW>(sh[warp], sl[warp], jn, jc, h1, l1, ii, a1);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) acc[0][d].x = a1[0][d];
+    } else {
+      if (diag)
+        segment_f32x2<I, true, UNITW>(sh[warp], sl[warp], jn, jc, nxh, nxl, ii, acc);
+      else
+        segment_f32x2<I, false, UNITW>(sh[warp], sl[warp], jn, jc, nxh, nxl, ii, acc);
+    }
+#pragma unroll
+    for (int k = 0; k < I; ++k)
+#pragma unroll
+      for (int d = 0; d < 3; ++d) s_sum[warp][d][32 * k + lane] = k ? acc[0][d].y : acc[0][d].x;
   }
-  if (!g_addr[dev]) return IONTRAP_ECUDA;
-  *out = g_addr[dev];
-  return IONTRAP_OK;
+  __syncthreads();
+  // the chunks' sums, Kahan-added in chunk order (the accumulators hold the negated sums)
+  for (int k = tid; k < 3 * kBlockIons; k += threads) {
+    float ks = 0.0f, kc = 0.0f;
+    for (int c = 0; c < chunks; ++c) {
+      const float y = (&s_sum[c][0][0])[k] - kc;
+      const float t = ks + y;
+      kc = (t - ks) - y;
+      ks = t;
+    }
+    (&s_sum[0][0][0])[k] = ks;
+    (&s_comp[0][0])[k] = kc;
+  }
+  cluster.sync();
+  // CTA r finishes its share of the ions: the S partials in range order
+  const int S = (int)gridDim.y, r = (int)cluster.block_rank(), per = (kBlockIons + S - 1) / S;
+  for (int k = tid; k < 3 * per; k += threads) {
+    const int c = k / per, q = r * per + (k - c * per), i = i0 + q;
+    if (q >= kBlockIons || i >= n) continue;
+    float su = 0.f, cu = 0.f, a[kNoAllocMaxSplits], b[kNoAllocMaxSplits];
+#pragma unroll
+    for (int p = 0; p < kNoAllocMaxSplits; ++p)
+      if (p < S) {
+        a[p] = *cluster.map_shared_rank(&s_sum[0][c][q], (unsigned)p);
+        b[p] = *cluster.map_shared_rank(&s_comp[c][q], (unsigned)p);
+      }
+#pragma unroll
+    for (int p = 0; p < kNoAllocMaxSplits; ++p)
+      if (p < S) kahan_merge(su, cu, a[p], b[p]);
+    A.out[(size_t)c * n + i] = A.coul[A.sp[i]] * (widen(cu) - widen(su));
+  }
+  cluster.sync();  // nobody leaves while others read its shared memory
 }
 
 }  // namespace
@@ -93,50 +165,36 @@ extern "C" int iontrap_forces_noalloc(const iontrap_species* species, int n_spec
       return IONTRAP_EINVAL;
   if (n > kNoAllocMaxIons) return IONTRAP_ETOOLARGE;
 
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return IONTRAP_ECUDA;
-  cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  unsigned char* base = nullptr;
-  const int st = scratch_for_device(dev, stream, &base);
-  if (st) return st;
-
-  StepArgs A{};
-  A.n = n;
-  float4* hi = reinterpret_cast<float4*>(base + kOffPair);
-  A.hi[0] = A.hi[1] = hi;
-  A.lo[0] = A.lo[1] = hi + n;
-  A.x = const_cast<double*>(d_x);
-  A.sp = d_species_of_ion;
-  A.part = base + kOffPart;
-  A.cnt = reinterpret_cast<unsigned*>(base + kOffCnt);
-  A.done = reinterpret_cast<unsigned*>(base + kOffDone);
-  A.step = reinterpret_cast<long long*>(base + kOffStep);
-  A.err = reinterpret_cast<int*>(base + kOffErr);
-  A.out = d_acc;
-  A.mode = MODE_FORCES;
-  const long long iblocks = (n + kNoAllocThreads - 1) / kNoAllocThreads;
+  ForcesArgs A{};
+  A.n = (int)n, A.sp = d_species_of_ion, A.x = d_x, A.out = d_acc;
+  // equal j-ranges of at least 128 ions, at most 8
   const long long splits = std::min<long long>(kNoAllocMaxSplits, std::max<long long>(1, (n + 127) / 128));
   A.jsplit = (int)((n + splits - 1) / splits);
-  A.nsplit = (int)((n + A.jsplit - 1) / A.jsplit);
+  const unsigned nsplit = (unsigned)((n + A.jsplit - 1) / A.jsplit);
   const double ke = 1.0 / (4.0 * kPi * kEps0);
+  bool unitw = true;
   for (int s = 0; s < n_species; ++s) {
     const double M = species[s].mass_amu * kAmu, z = species[s].charge_e;
-    A.spc[s].coul = ke * kE * kE * z / M;
-    A.spc[s].w = (float)z;
+    A.coul[s] = ke * kE * kE * z / M;
+    A.w[s] = (float)z;
+    unitw = unitw && z == 1.0;
   }
-
-  // step = 0, error flags = 0, done = 0, counters = 0; the output starts as NaN (all bits
-  // set), so an ion whose sum never completes -- its i-block gave up on a bounded wait --
-  // reads NaN instead of a stale value
-  cudaError_t e = cudaMemsetAsync(base, 0, kOffCnt + kCntBytes, stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d_acc, 0xFF, 3 * (size_t)n * sizeof(double), stream);
-  int b = 0, f64 = 0;
-  void* prep_params[] = {&A, &b, &f64};
-  const unsigned prep_blocks = (unsigned)std::min<long long>((n + 255) / 256, 4096);
-  if (e == cudaSuccess) e = cudaLaunchKernel(prep_kernel(), dim3(prep_blocks), dim3(256), prep_params, 0, stream);
-  void* params[] = {&A};
-  if (e == cudaSuccess)
-    e = cudaLaunchKernel(step_kernel(kNoAllocThreads, 1, 0, 1), dim3((unsigned)iblocks, (unsigned)A.nsplit),
-                         dim3(kNoAllocThreads), params, 0, stream);
+  cudaLaunchConfig_t cfg{};
+  // one ion per lane while the chip is short of warps (us per call, 1 / 2 ions per lane:
+  // n = 1000: 10.3 / 12.4, 3000: 16.3 / 16.5, 4097: 24.3 / 19.6, 8192: 62 / 55)
+  const int I = n <= 3200 ? 1 : 2;
+  cfg.gridDim = dim3((unsigned)((n + 32 * I - 1) / (32 * I)), nsplit);
+  cfg.blockDim = dim3(32u * (unsigned)((A.jsplit + kSeg - 1) / kSeg));
+  cfg.stream = static_cast<cudaStream_t>(cuda_stream);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 1;
+  attr[0].val.clusterDim.y = nsplit;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(
+      &cfg, I == 1 ? (unitw ? k_forces_cluster<1, true> : k_forces_cluster<1, false>)
+                   : (unitw ? k_forces_cluster<2, true> : k_forces_cluster<2, false>), A);
   return e == cudaSuccess ? IONTRAP_OK : IONTRAP_ECUDA;
 }

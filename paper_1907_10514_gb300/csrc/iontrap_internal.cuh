@@ -220,13 +220,22 @@ __device__ __forceinline__ void trace_mark(unsigned long long* trace, long long 
 }
 
 // ------------------------------------------------------------------ float <-> double
+// The conversions themselves, for the values the bit forms below leave.  Not inlined: as a few
+// predicated instructions they would hold the FP64 pipe ~70 cycles each for every warp, also
+// with no lane taking part (measured: 295 cycles per split_hilo so, ~40 with calls).
+static __device__ __noinline__ double cvt_f32_f64(float x) { return (double)x; }
+static __device__ __noinline__ float2 cvt_hilo(double x) {
+  const float hi = __double2float_rn(x);
+  return make_float2(hi, __double2float_rn(x - (double)hi));
+}
+
 // (double)x without the FP64-rate conversion: normal floats and zeros by their bits.
 __device__ __forceinline__ double widen(float x) {
   const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
   if (m - 0x00800000u < 0x7f000000u)  // normal
     return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
   if (m == 0u) return __hiloint2double((int)b, 0);
-  return (double)x;
+  return cvt_f32_f64(x);
 }
 
 // hi = fl(x), lo = fl(x - hi) without FP64-rate operations: the mantissa's top 24 bits
@@ -243,8 +252,8 @@ __device__ __forceinline__ void split_hilo(double x, float& hi, float& lo) {
     lo = __int2float_rn((xh >> 31) ? -r : r) * __uint_as_float((e - 948u) << 23);
     return;
   }
-  hi = __double2float_rn(x);
-  lo = __double2float_rn(x - (double)hi);
+  const float2 p = cvt_hilo(x);
+  hi = p.x, lo = p.y;
 }
 
 // ------------------------------------------------------------------ FP32 pair terms
@@ -280,36 +289,62 @@ __device__ __forceinline__ void segment_f32(const float4* __restrict__ sh, const
 // The same arithmetic on two ions per instruction (packed FP32x2 FADD/FMUL/FFMA of
 // sm_100+); each lane rounds exactly as the scalar loop does, so both loops give the
 // same bits.
+//
+// V consecutive j: all differences first, then the reciprocal roots, then the sums in j order.
+// A j's chain is ~100 cycles and a warp alone waited for most of it; written by stages over 16 j
+// (2 ions per thread) it takes 60 a j (4 warps of a sub-partition: 175 -> 160 for all four).
+template <int I, int V, bool DIAG, bool UNITW>
+__device__ __forceinline__ void group_f32x2(const float4* __restrict__ sh, const float4* __restrict__ sl, int j,
+                                            long long jbase, const float2 (&nxh)[I / 2][3],
+                                            const float2 (&nxl)[I / 2][3], const long long (&ii)[I],
+                                            float2 (&acc)[I / 2][3]) {
+  float2 d[V][I / 2][3], r[V][I / 2];
+  float w[V];
+#pragma unroll
+  for (int u = 0; u < V; ++u) {
+    const float4 ph = sh[j + u];
+    const float4 pl = sl[j + u];
+    const float2 h[3] = {make_float2(ph.x, ph.x), make_float2(ph.y, ph.y), make_float2(ph.z, ph.z)};
+    const float2 l[3] = {make_float2(pl.x, pl.x), make_float2(pl.y, pl.y), make_float2(pl.z, pl.z)};
+    w[u] = ph.w;
+#pragma unroll
+    for (int k = 0; k < I / 2; ++k) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) d[u][k][c] = __fadd2_rn(__fadd2_rn(h[c], nxh[k][c]), __fadd2_rn(l[c], nxl[k][c]));
+      r[u][k] = __ffma2_rn(d[u][k][0], d[u][k][0], __ffma2_rn(d[u][k][1], d[u][k][1], __fmul2_rn(d[u][k][2], d[u][k][2])));
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < V; ++u)
+#pragma unroll
+    for (int k = 0; k < I / 2; ++k) r[u][k] = make_float2(rsqrt_approx(r[u][k].x), rsqrt_approx(r[u][k].y));
+#pragma unroll
+  for (int u = 0; u < V; ++u)
+#pragma unroll
+    for (int k = 0; k < I / 2; ++k) {
+      float2 ri = r[u][k];
+      if (DIAG) {
+        ri.x = (jbase + j + u == ii[2 * k]) ? 0.0f : ri.x;
+        ri.y = (jbase + j + u == ii[2 * k + 1]) ? 0.0f : ri.y;
+      }
+      const float2 ri2 = __fmul2_rn(ri, ri);
+      const float2 s = __fmul2_rn(UNITW ? ri : __fmul2_rn(make_float2(w[u], w[u]), ri), ri2);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) acc[k][c] = __ffma2_rn(s, d[u][k][c], acc[k][c]);
+    }
+}
+
 template <int I, bool DIAG, bool UNITW = false>
 __device__ __forceinline__ void segment_f32x2(const float4* __restrict__ sh, const float4* __restrict__ sl, int jn,
                                               long long jbase, const float2 (&nxh)[I / 2][3],
                                               const float2 (&nxl)[I / 2][3], const long long (&ii)[I],
                                               float2 (&acc)[I / 2][3]) {
-#pragma unroll 4
-  for (int j = 0; j < jn; ++j) {
-    const float4 ph = sh[j];
-    const float4 pl = sl[j];
-    const float2 hx = make_float2(ph.x, ph.x), hy = make_float2(ph.y, ph.y), hz = make_float2(ph.z, ph.z);
-    const float2 lx = make_float2(pl.x, pl.x), ly = make_float2(pl.y, pl.y), lz = make_float2(pl.z, pl.z);
-    const float2 w = make_float2(ph.w, ph.w);
-#pragma unroll
-    for (int k = 0; k < I / 2; ++k) {
-      const float2 dx = __fadd2_rn(__fadd2_rn(hx, nxh[k][0]), __fadd2_rn(lx, nxl[k][0]));
-      const float2 dy = __fadd2_rn(__fadd2_rn(hy, nxh[k][1]), __fadd2_rn(ly, nxl[k][1]));
-      const float2 dz = __fadd2_rn(__fadd2_rn(hz, nxh[k][2]), __fadd2_rn(lz, nxl[k][2]));
-      const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-      float2 ri = make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
-      if (DIAG) {
-        ri.x = (jbase + j == ii[2 * k]) ? 0.0f : ri.x;
-        ri.y = (jbase + j == ii[2 * k + 1]) ? 0.0f : ri.y;
-      }
-      const float2 ri2 = __fmul2_rn(ri, ri);
-      const float2 s = __fmul2_rn(UNITW ? ri : __fmul2_rn(w, ri), ri2);
-      acc[k][0] = __ffma2_rn(s, dx, acc[k][0]);
-      acc[k][1] = __ffma2_rn(s, dy, acc[k][1]);
-      acc[k][2] = __ffma2_rn(s, dz, acc[k][2]);
-    }
-  }
+  constexpr int V = I == 2 ? 16 : 3;
+  int j = 0;
+#pragma unroll 1
+  for (; j + V <= jn; j += V) group_f32x2<I, V, DIAG, UNITW>(sh, sl, j, jbase, nxh, nxl, ii, acc);
+#pragma unroll 1
+  for (; j < jn; ++j) group_f32x2<I, 1, DIAG, UNITW>(sh, sl, j, jbase, nxh, nxl, ii, acc);
 }
 
 // ------------------------------------------------------------------ part-major pair loop
