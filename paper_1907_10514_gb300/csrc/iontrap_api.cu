@@ -1278,14 +1278,21 @@ int iontrap_hessian(iontrap_t* h, double* H) {
   DeviceGuard g(h->device);
   const size_t bytes = 9 * (size_t)h->n * (size_t)h->n * sizeof(double);
   double* d_H = nullptr;
-  if (cudaMalloc(&d_H, bytes) != cudaSuccess) return IONTRAP_ENOMEM;
+  // small matrices from the handles' pool, in order on the stream (cudaMalloc and cudaFree wait
+  // for the device); the pool would keep a large one
+  const bool pooled = bytes <= ((size_t)64 << 20);
+  if ((pooled ? dev_alloc(h, &d_H, bytes) : cudaMalloc(&d_H, bytes)) != cudaSuccess) return IONTRAP_ENOMEM;
   StepArgs a = h->args;
   if (h->p.flags & IONTRAP_COULOMB_OFF)
     for (int s = 0; s < IONTRAP_MAX_SPECIES; ++s) a.spc[s].z = 0.0;
   cudaError_t e = launch_hessian(a, d_H, h->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(H, d_H, bytes, cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  cudaFree(d_H);
+  const cudaError_t es = cudaStreamSynchronize(h->stream);
+  if (e == cudaSuccess) e = es;
+  if (pooled)
+    dev_free(h, d_H);
+  else
+    cudaFree(d_H);
   if (e != cudaSuccess) return cuda_status(h, e);
   return h->status;
 }

@@ -256,6 +256,62 @@ __device__ __forceinline__ void split_hilo(double x, float& hi, float& lo) {
   hi = p.x, lo = p.y;
 }
 
+// ------------------------------------------------------------------ FP64 inverse powers
+__device__ __forceinline__ double rsqrt_approx_f64(double x) {
+  double r;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  return __hiloint2double(__double2hiint(r), 0);
+}
+
+// y^2 of a double whose low word is zero: the 21-bit significand squared has at most 42 bits.
+// (y outside the normal range, or so small that y^2 is not normal, is squared by the FP64 pipe.)
+__device__ __forceinline__ double square21(double y) {
+  const unsigned h = (unsigned)__double2hiint(y);
+  const unsigned e = h >> 20;  // y >= 0
+  const unsigned m = (h & 0xfffffu) | 0x100000u;
+  const unsigned long long q = (unsigned long long)m * m;  // [2^40, 2^42)
+  const unsigned up = (unsigned)(q >> 41);
+  const unsigned long long f = (up ? q << 11 : q << 12) & 0xfffffffffffffull;
+  if (e - 520u > 1000u) return y * y;
+  return __longlong_as_double((long long)((unsigned long long)(2u * e - 1023u + up) << 52 | f));
+}
+
+// What r^-1, r^-2 and r^-3 are built from: y, the 21-bit approximation of r2^(-1/2), y^2 exactly,
+// e = 1 - r2 y^2 and e^2, of which 20 bits count, without the FP64 pipe (|e| below 2^-18, or
+// zero, or not a number; tiny e gives 0).
+struct InvParts {
+  double y, y2, e;
+  float e2;
+};
+__device__ __forceinline__ InvParts inv_parts(double r2) {
+  InvParts p;
+  p.y = rsqrt_approx_f64(r2);
+  p.y2 = square21(p.y);
+  p.e = __fma_rn(-r2, p.y2, 1.0);
+  const unsigned eh = (unsigned)__double2hiint(p.e) & 0x7fffffffu;
+  const float ef = eh > 0x39000000u ? __uint_as_float((eh - 0x38000000u) << 3) : 0.0f;
+  p.e2 = ef * ef;
+  return p;
+}
+// A float that is zero or normal, as a double by its bits.
+__device__ __forceinline__ double widen_normal(float q) {
+  const unsigned b = __float_as_uint(q);
+  return __hiloint2double(b ? (int)((b >> 3) + 0x38000000u) : 0, (int)(b << 29));
+}
+
+// r^-3 for r^2 = r2 (0 for an overflowed r^2, as 1 / infinity): y^3 (1 - e)^(-3/2).
+__device__ __forceinline__ double inv_cube(double r2, const InvParts& p) {
+  const double c = __fma_rn(1.5, p.e, widen_normal(1.875f * p.e2));
+  const double s = p.y2 * __fma_rn(p.y, c, p.y);
+  return __double2hiint(r2) == 0x7ff00000 ? 0.0 : s;
+}
+__device__ __forceinline__ double inv_cube(double r2) { return inv_cube(r2, inv_parts(r2)); }
+
+// r^-2: y^2 / (1 - e).
+__device__ __forceinline__ double inv_square(const InvParts& p) {
+  return __fma_rn(p.y2, p.e + widen_normal(p.e2), p.y2);
+}
+
 // ------------------------------------------------------------------ FP32 pair terms
 // d = x_j - x_i from hi/lo pairs, with the i side held negated in registers:
 // (x_j,hi - x_i,hi) is exact for close pairs (Sterbenz) and the lo difference restores

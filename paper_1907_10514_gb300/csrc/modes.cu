@@ -255,72 +255,66 @@ struct HessArgs {
   SpeciesDev spc[IONTRAP_MAX_SPECIES];
 };
 
-// Unweighted pair block d^2 (k_e e^2 z_i z_j / r) / dx_ia dx_jb for r = x_i - x_j.
-__device__ __forceinline__ void pair_block(const HessArgs& A, long long i, long long j, double h[3][3]) {
-  const long long n = A.n;
-  double r[3], r2 = 0.0;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    r[c] = A.x[c * n + i] - A.x[c * n + j];
-    r2 += r[c] * r[c];
-  }
-  const double rr = sqrt(r2);
-  const double r3 = r2 * rr, r5 = r3 * r2;
-  const double kq = A.ke2 * A.spc[A.sp[i]].z * A.spc[A.sp[j]].z;
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) h[a][b] = kq * ((a == b ? 1.0 : 0.0) / r3 - 3.0 * r[a] * r[b] / r5);
-}
+// A CTA per ion i, a thread per j: the row's off-diagonal blocks, and the diagonal block
+// from their sum (fixed order: j by threads, then a tree), plus the trap springs M_i k_a, over
+// M_i.  A pair block is kq (delta_ab r^-3 - 3 r_a r_b r^-5), symmetric, from r^-2 and r^-3
+// without a division or a root: ~36 FP64 instructions a pair, where eighteen divisions in
+// two kernels took ~500 (n = 300, with the copy to the host: 251 -> 79 us a call).
+constexpr int kHessThreads = 128;
 
-// Off-diagonal blocks: one thread per (i, j), j along x.
-__global__ void __launch_bounds__(128) k_hess_pairs(const __grid_constant__ HessArgs A) {
-  const long long n = A.n;
-  const long long i = blockIdx.y;
-  const long long j = blockIdx.x * 128LL + threadIdx.x;
-  if (j >= n || i >= n || i == j) return;
-  double h[3][3];
-  pair_block(A, i, j, h);
-  const double w = 1.0 / sqrt(A.spc[A.sp[i]].mass * A.spc[A.sp[j]].mass);
-  const long long m = 3 * n;
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) A.H[(3 * i + a) * m + 3 * j + b] = h[a][b] * w;
-}
-
-// Diagonal blocks: one CTA per ion i; minus the sum over j of the pair blocks (fixed
-// order tree), plus the trap springs M_i k_a, over M_i.
-__global__ void __launch_bounds__(128) k_hess_diag(const __grid_constant__ HessArgs A) {
-  __shared__ double sh[9][128];
-  const long long n = A.n;
-  const long long i = blockIdx.x;
-  double acc[9];
-#pragma unroll
-  for (int q = 0; q < 9; ++q) acc[q] = 0.0;
-  for (long long j = threadIdx.x; j < n; j += 128) {
-    if (j == i) continue;
-    double h[3][3];
-    pair_block(A, i, j, h);
-#pragma unroll
-    for (int q = 0; q < 9; ++q) acc[q] -= h[q / 3][q % 3];
+__global__ void __launch_bounds__(kHessThreads) k_hessian(const __grid_constant__ HessArgs A) {
+  __shared__ double sh[6][kHessThreads];
+  __shared__ double s_w[IONTRAP_MAX_SPECIES], s_kq[IONTRAP_MAX_SPECIES];
+  const long long n = A.n, m = 3 * n;
+  const int i = blockIdx.x, tid = threadIdx.x, si = A.sp[i];
+  if (tid < IONTRAP_MAX_SPECIES) {
+    s_w[tid] = 1.0 / sqrt(A.spc[si].mass * A.spc[tid].mass);
+    s_kq[tid] = A.ke2 * A.spc[si].z * A.spc[tid].z;
   }
-#pragma unroll
-  for (int q = 0; q < 9; ++q) sh[q][threadIdx.x] = acc[q];
   __syncthreads();
-  for (int w = 64; w > 0; w >>= 1) {
-    if (threadIdx.x < w)
+  const double xi[3] = {A.x[i], A.x[n + i], A.x[2 * n + i]};
+  double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};  // xx, yy, zz, xy, xz, yz
+  for (int j = tid; j < n; j += kHessThreads) {
+    if (j == i) continue;
+    double r[3];
 #pragma unroll
-      for (int q = 0; q < 9; ++q) sh[q][threadIdx.x] += sh[q][threadIdx.x + w];
+    for (int c = 0; c < 3; ++c) r[c] = xi[c] - A.x[c * n + j];
+    const int sj = A.sp[j];
+    const double r2 = __fma_rn(r[0], r[0], __fma_rn(r[1], r[1], r[2] * r[2]));
+    const InvParts p = inv_parts(r2);
+    const double k3 = s_kq[sj] * inv_cube(r2, p);
+    const double k5 = 3.0 * k3 * inv_square(p);
+    const double t[3] = {r[0] * k5, r[1] * k5, r[2] * k5};
+    const double b[6] = {__fma_rn(-t[0], r[0], k3), __fma_rn(-t[1], r[1], k3), __fma_rn(-t[2], r[2], k3),
+                         -t[0] * r[1], -t[0] * r[2], -t[1] * r[2]};
+    const double w = s_w[sj];
+    double o[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) acc[q] -= b[q], o[q] = b[q] * w;
+    double* H = A.H + 3LL * i * m + 3LL * j;
+    H[0] = o[0], H[1] = o[3], H[2] = o[4];
+    H[m] = o[3], H[m + 1] = o[1], H[m + 2] = o[5];
+    H[2 * m] = o[4], H[2 * m + 1] = o[5], H[2 * m + 2] = o[2];
+  }
+#pragma unroll
+  for (int q = 0; q < 6; ++q) sh[q][tid] = acc[q];
+  __syncthreads();
+  for (int w = kHessThreads / 2; w > 0; w >>= 1) {
+    // the six sums' halves over the CTA's threads
+    for (int u = tid; u < 6 * w; u += kHessThreads) {
+      const int q = u / w, k = u - q * w;
+      sh[q][k] += sh[q][k + w];
+    }
     __syncthreads();
   }
-  if (threadIdx.x < 9) {
-    const int a = threadIdx.x / 3, b = threadIdx.x % 3;
-    const SpeciesDev& sd = A.spc[A.sp[i]];
+  if (tid < 9) {
+    const int a = tid / 3, b = tid % 3;
+    const SpeciesDev& sd = A.spc[si];
     double k[3];
     trap_springs(A.trap, sd, 0.0, k);
-    const double d = sh[threadIdx.x][0] + (a == b ? sd.mass * k[a] : 0.0);
-    A.H[(3 * i + a) * (3 * n) + 3 * i + b] = d / sd.mass;
+    const int q = a == b ? a : a + b + 2;  // xy, xz, yz at 3, 4, 5
+    const double d = sh[q][0] + (a == b ? sd.mass * k[a] : 0.0);
+    A.H[(3LL * i + a) * m + 3LL * i + b] = d / sd.mass;
   }
 }
 
@@ -334,10 +328,7 @@ cudaError_t launch_hessian(const StepArgs& s, double* d_H, cudaStream_t st) {
   A.trap = s.trap;
   for (int k = 0; k < IONTRAP_MAX_SPECIES; ++k) A.spc[k] = s.spc[k];
   void* params[] = {&A};
-  cudaError_t e = cudaLaunchKernel((const void*)k_hess_pairs, dim3((unsigned)((s.n + 127) / 128), (unsigned)s.n),
-                                   dim3(128), params, 0, st);
-  if (e == cudaSuccess) e = cudaLaunchKernel((const void*)k_hess_diag, dim3((unsigned)s.n), dim3(128), params, 0, st);
-  return e;
+  return cudaLaunchKernel((const void*)k_hessian, dim3((unsigned)s.n), dim3(kHessThreads), params, 0, st);
 }
 
 }  // namespace it

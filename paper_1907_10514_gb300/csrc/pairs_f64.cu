@@ -67,42 +67,6 @@ struct F64Args {
 constexpr int kF64Threads = 128;
 constexpr int kF64NoiseIons = 16;  // ions of a noise unit (32 lanes: two numbers each)
 
-__device__ __forceinline__ double rsqrt_approx_f64(double x) {
-  double r;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  return __hiloint2double(__double2hiint(r), 0);
-}
-
-// y^2 of a double whose low word is zero: the 21-bit significand squared has at most 42 bits.
-// (y outside the normal range, or so small that y^2 is not normal, is squared by the FP64 pipe.)
-__device__ __forceinline__ double square21(double y) {
-  const unsigned h = (unsigned)__double2hiint(y);
-  const unsigned e = h >> 20;  // y >= 0
-  const unsigned m = (h & 0xfffffu) | 0x100000u;
-  const unsigned long long q = (unsigned long long)m * m;  // [2^40, 2^42)
-  const unsigned up = (unsigned)(q >> 41);
-  const unsigned long long f = (up ? q << 11 : q << 12) & 0xfffffffffffffull;
-  if (e - 520u > 1000u) return y * y;
-  return __longlong_as_double((long long)((unsigned long long)(2u * e - 1023u + up) << 52 | f));
-}
-
-// r^-3 for r^2 = r2 (0 for an overflowed r^2, as 1 / infinity).
-__device__ __forceinline__ double inv_cube(double r2) {
-  const double y = rsqrt_approx_f64(r2);
-  const double y2 = square21(y);
-  const double e = __fma_rn(-r2, y2, 1.0);
-  // 15/8 e^2 in FP32: e's high word as a float by its bits (|e| below 2^-18 or zero or NaN;
-  // tiny e gives 0)
-  const unsigned eh = (unsigned)__double2hiint(e) & 0x7fffffffu;
-  const float ef = eh > 0x39000000u ? __uint_as_float((eh - 0x38000000u) << 3) : 0.0f;
-  const float q = 1.875f * ef * ef;
-  const unsigned qb = __float_as_uint(q);
-  const double qd = __hiloint2double(qb ? (int)((qb >> 3) + 0x38000000u) : 0, (int)(qb << 29));
-  const double c = __fma_rn(1.5, e, qd);
-  const double s = y2 * __fma_rn(y, c, y);
-  return __double2hiint(r2) == 0x7ff00000 ? 0.0 : s;
-}
-
 // Rotations k0 <= k < k1 of one tile.  Row sub-block s starts at ion 32 (a I + s); the column
 // block is col.  d = col - a I: the sub-block s < d meets every column, s == d is the block
 // itself (rotations 1 .. 16, the last one by half of the lanes), s > d was met before as a
