@@ -19,8 +19,8 @@
 //   pair warps (14)  the part sums; a thread keeps its ion and takes every G-th part, and
 //                    each round of G parts is handed to the owners while the next one runs
 //
-// Measured (200 steps of 64 ions, GB300): 3.30 us per step in one CTA before, 1.21 here; 321
-// ions 3.72 on the grid, 3.2 here.  Where the 2500 cycles of a step of 64 ions go: stores'
+// Measured (200 steps of 64 ions, GB300): 3.30 us per step in one CTA before, 1.21 here; 150
+// ions 4.0 on the grid, 1.92 here.  Where the 2500 cycles of a step of 64 ions go: stores'
 // flight and pair items 800, merge 300, FP64 update 700, stores 300, the next step's FP64
 // terms 500.
 //
@@ -359,6 +359,7 @@ size_t rpc_smem_bytes(int Rc, int NPe, int JP, long long K) {
 //   n = 16: 2.84 / 1.15 1.07 - -      64: 3.30 / - 1.26 1.21 1.23    100: 4.97 / - 1.61 1.57 1.43
 //   128: 5.69 / - 2.05 1.73 1.53     200: 4.09 / - - 2.50 2.14       256: 4.13 / - - 3.06 2.58
 //   400: 3.49 / - - - 3.10           512: 3.51 / - - - 4.1
+// Above 168 ions most shapes are stepped by tagged_step.cu instead.
 int rpc_ctas(long long n, int JP) {
   if (JP > kSeg || n > kRpcMaxN) return 0;
   return n < 13 ? 1 : n < 29 ? 4 : n <= 84 ? 8 : 16;

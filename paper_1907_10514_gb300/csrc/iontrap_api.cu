@@ -53,6 +53,10 @@ cudaError_t launch_rp(const StepArgs& a, unsigned* sync, int W, int R, int NP, i
                       cudaStream_t st);
 int rp_max_ctas(int W, int R, int NP, int JP, int I, long long max_k, int sms);
 size_t rp_smem_bytes(int W, int R, int NP, int JP, long long K);
+size_t tag_bytes(long long n);
+bool tag_takes(long long n, int W, int R, int JP, int G, int sms, bool cluster);
+cudaError_t launch_tag(const StepArgs& a, unsigned* sync, unsigned* tags, int R, int JP, int I, int G,
+                       long long K, cudaStream_t st);
 // minimize.cu
 bool minimize_shape(long long n, int R, int NP, int JP, int sms, int* ctas, int* ions, bool* cluster);
 size_t minimize_scratch_bytes(long long n, int ctas);
@@ -129,7 +133,8 @@ struct iontrap {
   GpShape gp{};                 // fused = 4
   RpShape rp{};                 // fused = 5
   F64View f64v{};               // FP64 form: its scratch
-  unsigned* d_gsync = nullptr;  // fused = 4, 5: step and group counters (zero between launches)
+  // fused = 4, 5: step and group counters (zero between launches), then the tagged positions
+  unsigned* d_gsync = nullptr;
   double* d_snap = nullptr;     // iontrap_step_record: x_{s-W}, x_{s-W+1} [2][3][n]
   StepArgs args{};
   // graph of kGraphSteps chained steps
@@ -693,8 +698,9 @@ int alloc_scratch(iontrap* h) {
         !gp_shape(h->n, h->f64, h->p.flags, h->sms, h->T, h->I, h->packed, h->jsplit, &h->gp))
       return IONTRAP_EINVAL;
     if (!h->d_gsync) {
-      if (dev_alloc(h, &h->d_gsync, kGpSyncBytes) != cudaSuccess) return IONTRAP_ENOMEM;
-      if (cudaMemsetAsync(h->d_gsync, 0, kGpSyncBytes, h->stream) != cudaSuccess) return IONTRAP_ECUDA;
+      const size_t bytes = kGpSyncBytes + tag_bytes(h->n);
+      if (dev_alloc(h, &h->d_gsync, bytes) != cudaSuccess) return IONTRAP_ENOMEM;
+      if (cudaMemsetAsync(h->d_gsync, 0, bytes, h->stream) != cudaSuccess) return IONTRAP_ECUDA;
     }
   }
   if (h->f64 && f64_prepare(h->n, h->sms, h->d_part, h->stream, &h->f64v) != cudaSuccess) return IONTRAP_ECUDA;
@@ -709,10 +715,15 @@ int alloc_scratch(iontrap* h) {
 
 // One row-persistent launch of K steps on the handle's buffers.
 cudaError_t launch_rp_of(iontrap* h, const StepArgs& a, long long K, cudaStream_t st) {
-  // steps of a small simulation run on one cluster (same bits); force evaluations, traced
-  // launches and those of the failure test, which look at the grid's counter, do not
-  if (a.mode == MODE_STEP && !a.trace && !a.stall_on && !a.wait_ns) {
-    const int C = rpc_ctas(h->n, h->rp.JP);
+  // steps of a small simulation run on one cluster, those of the next sizes on the grid with
+  // tagged positions (the same bits all three); force evaluations and launches of the failure
+  // test, which look at the grid's counter, do not, and traced launches, marked per CTA of the
+  // grid, keep off the cluster
+  if (a.mode == MODE_STEP && !a.stall_on && !a.wait_ns) {
+    const int C = a.trace ? 0 : rpc_ctas(h->n, h->rp.JP);
+    if (tag_takes(h->n, h->rp.W, h->rp.R, h->rp.JP, h->rp.G, h->sms, C > 0))
+      return launch_tag(a, h->d_gsync, h->d_gsync + kGpSyncBytes / sizeof(unsigned), h->rp.R, h->rp.JP, h->rp.I,
+                        h->rp.G, K, st);
     if (C > 0) return launch_rpc(a, h->nspecies, C, h->rp.JP, K, st);
   }
   return launch_rp(a, h->d_gsync, h->rp.W, h->rp.R, h->rp.NP, h->rp.JP, h->rp.I, h->rp.G, K, st);
@@ -1611,7 +1622,7 @@ int iontrap_estimate_bytes(int64_t n, int precision, int64_t* bytes) {
   const int64_t vec = 3 * n * (int64_t)sizeof(double);
   const int64_t pair = n * (int64_t)(f64 ? sizeof(double4_32a) : 2 * sizeof(float4));
   *bytes = 3 * vec + n + 2 * pair + part + iblocks * (int64_t)sizeof(unsigned) + 64 +
-           (F >= 4 ? (int64_t)kGpSyncBytes : 0);
+           (F >= 4 ? (int64_t)(kGpSyncBytes + tag_bytes(n)) : 0);
   return IONTRAP_OK;
 }
 
@@ -1900,7 +1911,8 @@ int iontrap_device_bytes(const iontrap_t* h, int64_t* bytes) {
   const int64_t vec = 3 * h->n * (int64_t)sizeof(double);
   const int64_t pair = h->n * (int64_t)(h->f64 ? sizeof(double4_32a) : 2 * sizeof(float4));
   *bytes = 3 * vec + (h->d_out ? vec : 0) + (h->d_snap ? 2 * vec : 0) + h->n + 2 * pair + (int64_t)h->part_bytes +
-           (int64_t)h->cnt_len * (int64_t)sizeof(unsigned) + 64 + (h->d_gsync ? (int64_t)kGpSyncBytes : 0);
+           (int64_t)h->cnt_len * (int64_t)sizeof(unsigned) + 64 +
+           (h->d_gsync ? (int64_t)(kGpSyncBytes + tag_bytes(h->n)) : 0);
   return IONTRAP_OK;
 }
 
