@@ -315,7 +315,8 @@ typedef struct {
     int32_t jsplit;           /* j-range per CTA: grid.y = ceil(n / jsplit) */
     int32_t fused;            /* how the split partials are merged and integrated:
                                  1: by the last CTA of each i-block (arrival counter);
-                                 0: by a separate epilogue kernel over all SMs;
+                                 0: by a separate epilogue kernel over all SMs, a thread per
+                                    ion component (with pdl it waits beside the pair CTAs);
                                  2: the splits of an i-block form a thread-block cluster
                                     (at most 8 splits; 16 in form 3) and merge through distributed shared
                                     memory, each CTA integrating a slice of the i-block;

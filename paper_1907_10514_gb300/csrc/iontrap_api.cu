@@ -28,7 +28,7 @@ bool batched_shape_fits(long long n, int C, int NP);
 cudaError_t launch_batched(const std::vector<BatchEns>& ens, const std::vector<long long>& steps, int K,
                            cudaStream_t stream);
 const void* step_kernel(int T, int I, int packed, int fused);
-const void* epilogue_kernel();
+const void* epilogue_kernel(int* ions, int* threads);
 cudaError_t allow_large_clusters();
 const void* prep_kernel();
 const void* restore_kernel();
@@ -415,10 +415,11 @@ void default_config(int64_t n, int f64, int sms, int* T, int* I, int* packed, in
   if (!*fused && cdiv(n, js) > kMaxSplitsUnfused) js = cdiv(n, kMaxSplitsUnfused);
   *jsplit = (int)js;
   // above 8192: j-ranges laid out for blocks of 512 ions, summed by CTAs of 64 threads and 2
-  // ions each (the same bits: they depend on the j-ranges only).  Eight times the CTAs, and
-  // the last of an i-block integrates 128 ions instead of 512 (us per step, 128 x 4 against
-  // 64 x 2: n = 9001: 84 -> 64, 16384: 183 -> 153, 32768: 654 -> 564)
-  if (!f64 && n > 8192) *T = 64, *I = 2;
+  // ions each (the same bits: they depend on the j-ranges only), eight times the CTAs; and
+  // merged by the epilogue kernel, launched ahead of its sums (us per step, 128 x 4 / 64 x 2
+  // finished by the last CTA of an i-block, two warps that take 12 us for it / 64 x 2 and the
+  // epilogue kernel: n = 9001: 84 / 62 / 51, 16384: 183 / 150 / 140, 32768: 654 / 546 / 537)
+  if (!f64 && n > 8192) *T = 64, *I = 2, *fused = 0;
   // 2048 < n <= 8192: the cluster + warp-split form (4 warps, 2 ions per lane, 8-CTA
   // clusters) measured fastest (20.8 us/step at n = 4096 against 24.7 for the others)
   if (!f64 && n > 2048 && n <= 8192) {
@@ -769,10 +770,12 @@ cudaError_t launch_step_on(iontrap* h, StepArgs& a, cudaStream_t st) {
   void* params[] = {&a};
   cudaError_t e = cudaLaunchKernelExC(&cfg, step_kernel(h->T, h->I, h->packed, h->fused), params);
   if (e != cudaSuccess || h->fused != 0) return e;
-  cfg.gridDim = dim3((unsigned)cdiv(h->n, 32));  // 32 ions per epilogue CTA
-  cfg.blockDim = dim3(256);
+  int ions, threads;
+  const void* epi = epilogue_kernel(&ions, &threads);
+  cfg.gridDim = dim3((unsigned)cdiv(h->n, ions));
+  cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = 0;
-  return cudaLaunchKernelExC(&cfg, epilogue_kernel(), params);
+  return cudaLaunchKernelExC(&cfg, epi, params);
 }
 
 cudaError_t launch_mode(iontrap* h, int mode, double* out) {
@@ -971,6 +974,7 @@ int iontrap_create(const iontrap_species* species, int n_species, const uint8_t*
     h->own_stream = true;
   }
   default_config(n, h->f64, h->sms, &h->T, &h->I, &h->packed, &h->jsplit, &h->fused);
+  h->pdl = h->fused == 0;
   if ((p->flags & IONTRAP_COULOMB_OFF) && h->fused >= 2) {  // cluster forms need the pair term
     h->T = 64, h->I = 1, h->packed = 0, h->fused = 1;
   }
@@ -1469,7 +1473,9 @@ int iontrap_trace_step(iontrap_t* h, unsigned long long* marks, int64_t cap, int
   }
   const dim3 grid = grid_of(h);
   const int64_t nf = 4 * (int64_t)grid.x * grid.y;
-  const int64_t ne = h->fused ? 0 : 2 * cdiv(h->n, 32);
+  int ions, threads;
+  epilogue_kernel(&ions, &threads);
+  const int64_t ne = h->fused ? 0 : 2 * cdiv(h->n, ions);
   if (nf + ne > cap) return IONTRAP_EINVAL;
   unsigned long long* d = nullptr;
   if (cudaMalloc(&d, (nf + ne) * sizeof(unsigned long long)) != cudaSuccess) return IONTRAP_ENOMEM;
@@ -1671,7 +1677,7 @@ int iontrap_autotune(iontrap_t* h, double trial_us, iontrap_config* best, double
       for (int fused = 2; fused >= 0; --fused) {
         if (fused == 2 && (cdiv(n, js) > kMaxClusterSplits || (h->p.flags & IONTRAP_COULOMB_OFF))) continue;
         if (!fused && cdiv(n, js) > kMaxSplitsUnfused) continue;
-        iontrap_config c{sh.T, sh.I, sh.P, (int32_t)js, fused, 0, 1};
+        iontrap_config c{sh.T, sh.I, sh.P, (int32_t)js, fused, fused == 0, 1};
         if (step_kernel(c.threads, c.ions_per_thread, c.packed, c.fused)) cands.push_back(c);
       }
     }
@@ -1927,7 +1933,7 @@ int iontrap_default_config(int64_t n, int precision, uint32_t flags, int allow_p
   default_config(n, precision == IONTRAP_PREC_FP64, sms, &c->threads, &c->ions_per_thread, &c->packed, &c->jsplit,
                  &c->fused, (flags & IONTRAP_COULOMB_OFF) ? 0 : allow_persistent);
   if ((flags & IONTRAP_COULOMB_OFF) && c->fused >= 2) c->threads = 64, c->ions_per_thread = 1, c->packed = 0, c->fused = 1;
-  c->pdl = 0;
+  c->pdl = c->fused == 0;
   c->graph = 1;
   return IONTRAP_OK;
 }

@@ -188,8 +188,11 @@ __device__ __forceinline__ bool pair_sums(const StepArgs& A, float4 (&sh)[2][kCh
   return true;
 }
 
+// The bound of one CTA per SM keeps ptxas from saving registers in small CTAs: it undid the staging
+// of the two-ion loop to fit more of them (64 threads, n = 32768: 71 registers and 662 us per
+// step, 106 and 537 with the bound).
 template <int T, int I, bool PACK, bool FUSED>
-__global__ void __launch_bounds__(T) k_step_f32(const __grid_constant__ StepArgs A) {
+__global__ void __launch_bounds__(T, 1) k_step_f32(const __grid_constant__ StepArgs A) {
   __shared__ __align__(128) float4 sh[2][kChunk];
   __shared__ __align__(128) float4 sl[2][kChunk];
   __shared__ __align__(8) uint64_t bar[2];
@@ -198,6 +201,7 @@ __global__ void __launch_bounds__(T) k_step_f32(const __grid_constant__ StepArgs
   __shared__ double s_springs[IONTRAP_MAX_SPECIES][3];
 
   pdl_wait();
+  if constexpr (!FUSED) pdl_trigger();  // the epilogue's CTAs: they need no sums at first
   const int tid = threadIdx.x;
   const long long n = A.n;
   const long long i0 = (long long)blockIdx.x * (T * I);
@@ -219,6 +223,20 @@ __global__ void __launch_bounds__(T) k_step_f32(const __grid_constant__ StepArgs
   if (!pair_sums<T, I, PACK>(A, sh, sl, bar, ghi, glo, i0, j0, j1, ks, kc)) return;
 
   trace_mark(A.trace, tslot + 1);
+  if constexpr (!FUSED) {  // the epilogue kernel merges the partials
+    float* part = reinterpret_cast<float*>(A.part) + 6 * n * blockIdx.y;
+#pragma unroll
+    for (int k = 0; k < I; ++k) {
+      const long long i = i0 + k * T + tid;
+      if (i < n)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          __stcg(part + c * n + i, ks[k][c]);
+          __stcg(part + (3 + c) * n + i, kc[k][c]);
+        }
+    }
+    return;
+  }
   pdl_trigger();  // dependents launch as the last CTAs finish their pair loops
   float4* part = reinterpret_cast<float4*>(A.part);
 #pragma unroll
@@ -230,7 +248,6 @@ __global__ void __launch_bounds__(T) k_step_f32(const __grid_constant__ StepArgs
       __stcg(part + r + 1, make_float4(kc[k][0], kc[k][1], kc[k][2], 0.0f));
     }
   }
-  if constexpr (!FUSED) return;  // the epilogue kernel merges the partials
   if (!arrive_last(&A.cnt[blockIdx.x], gridDim.y, &s_flag)) return;
   trace_mark(A.trace, tslot + 2);
 
@@ -605,82 +622,115 @@ __global__ void __launch_bounds__(32 * W) k_step_f32_cw(const __grid_constant__ 
   }
 }
 
-// Separate epilogue over all SMs.  A CTA of 256 threads serves 32 ions: 8 lanes per ion
-// fetch the ion's split records together (one memory round trip instead of one per
-// split), fold them in split order through warp shuffles, and leave the merged sum in
-// shared memory; then one warp integrates the 32 ions, one per lane.  The last CTA
-// advances the step counter.
-constexpr int kEpiIons = 32;
-constexpr int kEpiThreads = 256;
-constexpr int kEpiMaxRec = 8;  // records per lane: splits up to 8 * 8 = 64
+// Separate epilogue over all SMs: a thread per ion component (a CTA of 64 ions, warps of one
+// component), so that the FP64 update, whose instructions hold their pipe for ~76 cycles whatever
+// the active lanes, runs with full warps on every SM.
+//
+// State, noise, trap and laser terms do not depend on the pair sums: they are evaluated before
+// griddepcontrol.wait, while the pair grid runs.  The pair grid lets this one launch once all its
+// CTAs have passed their own wait, so the previous step's epilogue is complete by then.  The
+// partial sums lie as rows of n floats (six per split): each warp reads whole sectors.
+//
+// What bounds it: latencies, the loads of up to eight splits at a time, the Kahan chain and five
+// dependent FP64 operations, ~2 us after the pair grid's end.  n = 9001, 25 splits, us per step:
+// 62 when the last CTA of an i-block finished its 128 ions (two warps, 12 us), 68 with an epilogue
+// of four active lanes a warp after the pair grid, 51 here.
+constexpr int kEpiIons = 64;
+constexpr int kEpiThreads = 3 * kEpiIons;
+constexpr int kEpiBatch = 8;  // splits in flight
 
 __global__ void __launch_bounds__(kEpiThreads) k_epilogue_f32(const __grid_constant__ StepArgs A) {
   __shared__ double s_cos;
   __shared__ double s_springs[IONTRAP_MAX_SPECIES][3];
-  __shared__ int s_last;
-  pdl_wait();
+  __shared__ double s_vd[3][kEpiIons];
+  const int tid = threadIdx.x, c = tid / kEpiIons, q = tid - c * kEpiIons;
   const long long n = A.n;
+  const long long i = blockIdx.x * (long long)kEpiIons + q;
+  const bool on = i < n;
+  const TrapDev& tp = A.trap;
+  const bool step = A.mode == MODE_STEP, forces = A.mode == MODE_FORCES;
+  pdl_trigger();
   const long long ns = *A.step;
-  const int rb = (A.mode == MODE_STEP) ? (int)((ns + 1) & 1) : (int)(ns & 1);
+  const int wb = step ? (int)(ns & 1) : (int)((ns + 1) & 1);
+  const SpeciesDev& sd = A.spc[on ? A.sp[i] : 0];
+  double xf = 0.0, v0 = 0.0, vd = 0.0, ext = 0.0;
+  if (!forces) {
+    if (tid == 0) s_cos = force_time_cos(A, ns);
+    if (on) {
+      xf = A.x[c * n + i], v0 = A.v[c * n + i];
+      vd = half_kick(v0, A.a[c * n + i], tp.hdt);
+      if (step)
+        xf = drift(xf, vd, tp.dt);
+      else
+        vd = v0;
+    }
+    s_vd[c][q] = vd;
+    float z[3] = {0.f, 0.f, 0.f};
+    if (on && sd.sigma > 0.0) normals3_f32(tp.seed, step ? ns + 1 : ns, i, z);
+    __syncthreads();  // s_cos, s_vd
+    if (tid < IONTRAP_MAX_SPECIES) trap_springs(tp, A.spc[tid], s_cos, s_springs[tid]);
+    __syncthreads();
+    if (on) {  // the operations and order of accel_ext
+      ext = __fma_rn(-sd.gamma, vd, __dmul_rn(-s_springs[A.sp[i]][c], xf));
+      if (sd.lrate != 0.0) {
+        const double v3[3] = {s_vd[0][q], s_vd[1][q], s_vd[2][q]};
+        ext = __fma_rn(-laser_proj(sd, v3), sd.kdir[c], ext);
+      }
+      if (sd.sigma > 0.0) ext = __fma_rn(sd.sigma, widen(c == 0 ? z[0] : c == 1 ? z[1] : z[2]), ext);
+    }
+  }
+  pdl_wait();
   unsigned long long* et = A.trace ? A.trace + A.trace_epi : nullptr;
   trace_mark(et, 2ll * blockIdx.x);
-  if (threadIdx.x == 0) s_cos = force_time_cos(A, ns);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int sub = lane & 7;                       // lane within the ion's group of 8
-  const int slot = warp * 4 + (lane >> 3);        // ion slot in this CTA
-  const long long i = blockIdx.x * (long long)kEpiIons + slot;
-  const int nsplit = A.nsplit;
-  const float4* __restrict__ part = reinterpret_cast<const float4*>(A.part);
-  float4 ra[kEpiMaxRec], rc[kEpiMaxRec];
+  if (on) {
+    // the splits' sums and compensations of this component, merged in split order
+    const float* __restrict__ p = reinterpret_cast<const float*>(A.part) + c * n + i;
+    float su = 0.f, cu = 0.f;
+#pragma unroll 1
+    for (int p0 = 0; p0 < A.nsplit; p0 += kEpiBatch) {
+      float a[kEpiBatch], b[kEpiBatch];
 #pragma unroll
-  for (int q = 0; q < kEpiMaxRec; ++q) {
-    const int p = q * 8 + sub;
-    ra[q] = rc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (i < n && p < nsplit) {
-      ra[q] = __ldcg(part + 2 * (p * n + i));
-      rc[q] = __ldcg(part + 2 * (p * n + i) + 1);
+      for (int u = 0; u < kEpiBatch; ++u)
+        if (p0 + u < A.nsplit) {
+          a[u] = __ldcg(p + 6 * n * (p0 + u));
+          b[u] = __ldcg(p + 6 * n * (p0 + u) + 3 * n);
+        }
+#pragma unroll
+      for (int u = 0; u < kEpiBatch; ++u)
+        if (p0 + u < A.nsplit) kahan_merge(su, cu, a[u], b[u]);
     }
-  }
-  float s[3] = {0.f, 0.f, 0.f}, cc[3] = {0.f, 0.f, 0.f};
-  const int base = lane & ~7;
-#pragma unroll
-  for (int q = 0; q < kEpiMaxRec; ++q) {
-    if (q * 8 >= nsplit) break;
-#pragma unroll
-    for (int l = 0; l < 8; ++l) {
-      const int p = q * 8 + l;  // uniform across the warp
-      const float ax = __shfl_sync(0xffffffffu, ra[q].x, base + l), ay = __shfl_sync(0xffffffffu, ra[q].y, base + l);
-      const float az = __shfl_sync(0xffffffffu, ra[q].z, base + l), cx = __shfl_sync(0xffffffffu, rc[q].x, base + l);
-      const float cy = __shfl_sync(0xffffffffu, rc[q].y, base + l), cz = __shfl_sync(0xffffffffu, rc[q].z, base + l);
-      if (p < nsplit) {
-        kahan_merge(s[0], cc[0], ax, cx);
-        kahan_merge(s[1], cc[1], ay, cy);
-        kahan_merge(s[2], cc[2], az, cz);
+    const double S = widen(cu) - widen(su);
+    if (forces) {
+      A.out[c * n + i] = sd.coul * S;
+    } else {
+      const double acc = __fma_rn(sd.coul, S, ext);
+      const double vn = step ? half_kick(vd, acc, tp.hdt) : v0;
+      const double xn = drift(xf, half_kick(vn, acc, tp.hdt), tp.dt);
+      float h, l;
+      split_hilo(xn, h, l);
+      if (step) {
+        A.x[c * n + i] = xf;
+        A.v[c * n + i] = vn;
       }
+      A.a[c * n + i] = acc;
+      reinterpret_cast<float*>(A.hi[wb] + i)[c] = h;
+      reinterpret_cast<float*>(A.lo[wb] + i)[c] = l;
+      if (c == 0) {
+        reinterpret_cast<float*>(A.hi[wb] + i)[3] = sd.w;
+        reinterpret_cast<float*>(A.lo[wb] + i)[3] = 0.0f;
+      }
+      // a non-finite acceleration or velocity reaches xn = xf + dt (vn + dt/2 acc)
+      if ((((unsigned)__double2hiint(xn) >> 20) & 0x7ffu) == 0x7ffu) atomicOr(A.err, ERR_NONFINITE);
     }
   }
-  pdl_trigger();
-  __syncthreads();  // s_cos
-  if (threadIdx.x < IONTRAP_MAX_SPECIES) trap_springs(A.trap, A.spc[threadIdx.x], s_cos, s_springs[threadIdx.x]);
   __syncthreads();
-  // one lane per ion integrates; the 32 ions are spread over the 8 warps (4 per warp)
-  if (sub == 0 && i < n) {
-    double S[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) S[c] = (double)cc[c] - (double)s[c];
-    epilogue_ion<false>(A, i, S, s_springs, ns, rb ^ 1);
-  }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const unsigned prev = atomicAdd(A.done, 1u);
-    s_last = (prev == gridDim.x - 1u);
-  }
-  __syncthreads();
-  if (s_last && threadIdx.x == 0) {
-    *A.done = 0u;
-    if (A.mode == MODE_STEP) *A.step = ns + 1;
+  if (tid == 0) {  // the last CTA advances the step counter
     __threadfence();
+    if (atomicAdd(A.done, 1u) == gridDim.x - 1u) {
+      *A.done = 0u;
+      if (step) *A.step = ns + 1;
+      __threadfence();
+    }
   }
   trace_mark(et, 2ll * blockIdx.x + 1);
 }
@@ -770,7 +820,10 @@ cudaError_t allow_large_clusters() {
   return cudaSuccess;
 }
 
-const void* epilogue_kernel() { return (const void*)k_epilogue_f32; }
+const void* epilogue_kernel(int* ions, int* threads) {
+  *ions = kEpiIons, *threads = kEpiThreads;
+  return (const void*)k_epilogue_f32;
+}
 
 const void* prep_kernel() { return (const void*)k_prep; }
 const void* restore_kernel() { return (const void*)k_restore; }
