@@ -355,7 +355,8 @@ typedef struct {
                                  once in a layout that is a function of n, and threads,
                                  ions_per_thread and jsplit do not change its results. */
     int32_t pdl;              /* 1: consecutive step kernels use programmatic dependent launch
-                                 (default 0: measured slower on GB300 for these grids) */
+                                 (default: 1 with fused = 0, whose epilogue then starts while
+                                 the pairs are summed; otherwise 0, measured slower on GB300) */
     int32_t graph;            /* 1: iontrap_step enqueues CUDA graphs of 100 steps; 0: single launches */
 } iontrap_config;
 
