@@ -385,14 +385,14 @@ __global__ void __launch_bounds__(kBRThreads, 2)
           const bool diag = __any_sync(__activemask(), (jc < r0 + Rg) && (r0 < jc + qn));
           if (unitw) {
             if (diag)
-              rp_chunk<true, true>(sj + c0, sw + c0, JP, qn, jc, i, nh, nl, acc);
+              rp_chunk<true, true, 4>(sj + c0, sw + c0, JP, qn, jc, i, nh, nl, acc);
             else
-              rp_chunk<false, true>(sj + c0, sw + c0, JP, qn, jc, i, nh, nl, acc);
+              rp_chunk<false, true, 4>(sj + c0, sw + c0, JP, qn, jc, i, nh, nl, acc);
           } else {
             if (diag)
-              rp_chunk<true, false>(sj + c0, sw + c0, JP, qn, jc, i, nh, nl, acc);
+              rp_chunk<true, false, 4>(sj + c0, sw + c0, JP, qn, jc, i, nh, nl, acc);
             else
-              rp_chunk<false, false>(sj + c0, sw + c0, JP, qn, jc, i, nh, nl, acc);
+              rp_chunk<false, false, 4>(sj + c0, sw + c0, JP, qn, jc, i, nh, nl, acc);
           }
 #pragma unroll
           for (int d = 0; d < 3; ++d) {

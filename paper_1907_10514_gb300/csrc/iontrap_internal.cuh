@@ -434,11 +434,15 @@ __device__ __forceinline__ void rp_pair2(float2 hx, float2 hy, float2 hz, float2
 // y_lo, z_lo; the charges z from sw), four j per iteration from 16-byte shared loads.
 // Padding entries sit at 1e30 m: r^2 overflows to infinity, rsqrt gives 0, the term is
 // exactly 0.
-template <bool DIAG, bool UNITW>
+// U iterations at a time: with two warps in a sub-partition a chain of ~100 cycles shows (cycles
+// per iteration and warp, unrolled 2 / 4: one warp 106 / 89, two 89 / 77, four 78 / 76; 68 is the
+// packed pipe's), so the callers with two take 4 (us per step: n = 1000: 3.12 -> 2.99, 2047:
+// 5.34 -> 5.08); the row-persistent form's 16 warps lose to the remainder (n = 2500: 7.55 -> 7.87).
+template <bool DIAG, bool UNITW, int U = 2>
 __device__ __forceinline__ void rp_chunk(const float* __restrict__ sj, const float* __restrict__ sw, int JP, int qn,
                                          int jbase, int i, const float2 (&nh)[3], const float2 (&nl)[3],
                                          float2 (&acc)[3]) {
-#pragma unroll 2
+#pragma unroll U
   for (int q = 0; q < qn; q += 4) {
     const float4 hx = *reinterpret_cast<const float4*>(sj + q);
     const float4 hy = *reinterpret_cast<const float4*>(sj + JP + q);

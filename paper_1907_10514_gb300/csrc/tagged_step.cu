@@ -9,7 +9,7 @@
 // memory while the rest is awaited.  Two buffers alternate: who writes tag t + 2 has read all of
 // t + 1, whose writers had read all of t.
 //
-// What bounds a step (n = 1000, GB300, us: 3.88 before, 3.1 now): the handover, 0.9 from the last
+// What bounds a step (n = 1000, GB300, us: 3.88 before, 3.0 now): the handover, 0.9 from the last
 // store to the last arrival, of which the 32 n bytes that each of the G CTAs reads from L2 are
 // half (0.7 at n = 500, 1.25 at 2047); the pairs 1.0; the merge of the parts 0.35 (a Kahan
 // addition is a chain of four); the FP64 update and its stores 0.4.  Everything else is off the
@@ -25,8 +25,8 @@
 //
 // us per step (5 handles, K = 1000 steps a launch, this kernel / the counter and bulk copies;
 // below 432 ions / one cluster): n = 150: 2.01 / 1.92, 176: 2.02 / 2.04, 224: 2.16 / 2.31, 321:
-// 2.53 / 3.27, 432: 2.24 / 3.26, 500: 2.27 / 3.50, 800: 2.53 / 3.86, 1000: 3.1 / 3.89, 1500:
-// 3.57 / 4.39, 2047: 5.38 / 5.64.  With 16 warps a CTA (n > 2047) there was no gain: 2500: 7.70 /
+// 2.53 / 3.27, 432: 2.24 / 3.26, 500: 2.30 / 3.50, 800: 2.5 / 3.86, 1000: 3.0 / 3.89, 1500:
+// 3.54 / 4.39, 2047: 5.08 / 5.64.  With 16 warps a CTA (n > 2047) there was no gain: 2500: 7.70 /
 // 7.53, 3000: 8.5 / 8.6.
 //
 // The bits are those of persistent.cu's kernel for the same (n, NP, JP): the same part sums
@@ -251,14 +251,14 @@ __global__ void __launch_bounds__(kTagThreads, 1) k_step_f32_tag(const __grid_co
       if constexpr (IPT == 1) {
         if (A.unitw) {
           if (diag)
-            rp_chunk<true, true>(sj, sj + 6 * JP, JP, JP, jc, ii, nh[0], nl[0], acc[0]);
+            rp_chunk<true, true, 4>(sj, sj + 6 * JP, JP, JP, jc, ii, nh[0], nl[0], acc[0]);
           else
-            rp_chunk<false, true>(sj, sj + 6 * JP, JP, JP, jc, ii, nh[0], nl[0], acc[0]);
+            rp_chunk<false, true, 4>(sj, sj + 6 * JP, JP, JP, jc, ii, nh[0], nl[0], acc[0]);
         } else {
           if (diag)
-            rp_chunk<true, false>(sj, sj + 6 * JP, JP, JP, jc, ii, nh[0], nl[0], acc[0]);
+            rp_chunk<true, false, 4>(sj, sj + 6 * JP, JP, JP, jc, ii, nh[0], nl[0], acc[0]);
           else
-            rp_chunk<false, false>(sj, sj + 6 * JP, JP, JP, jc, ii, nh[0], nl[0], acc[0]);
+            rp_chunk<false, false, 4>(sj, sj + 6 * JP, JP, JP, jc, ii, nh[0], nl[0], acc[0]);
         }
       } else {
         if (A.unitw) {
