@@ -98,7 +98,16 @@ struct RpShape {
 };
 static constexpr int64_t kRpInitJsplit = 512;  // j-range per CTA of its creation-time / force evaluation
 
+// Counts the handles; the last one to go gives staging memory back (see Staging).
+struct LiveHandle {
+  LiveHandle();
+  ~LiveHandle();
+  LiveHandle(const LiveHandle&) = delete;
+  LiveHandle& operator=(const LiveHandle&) = delete;
+};
+
 struct iontrap {
+  LiveHandle live;
   int64_t n = 0;
   int nspecies = 0;
   iontrap_species species[IONTRAP_MAX_SPECIES]{};
@@ -594,12 +603,14 @@ constexpr size_t kHeaderBytes = 64;
 
 // Pinned host memory for the copies of small states: a driver call and a wait cost ~10 us each
 // on GB300, the copy of a few hundred KB through pinned memory less.  Buffers are kept for the
-// next call, at most kStagingKeep of them, none above kStagingMax bytes; p is null where the
-// copy is larger (or none can be had) and goes straight to and from the caller's arrays.
+// next call, at most kStagingKeep of them, one when no handle is left, none above kStagingMax
+// bytes; p is null where the copy is larger (or none can be had) and goes straight to and from
+// the caller's arrays.
 constexpr size_t kStagingMax = 256 * 1024;
 constexpr size_t kStagingKeep = 16;
 std::mutex g_staging_mu;
 std::vector<char*> g_staging;
+int g_handles = 0;
 
 struct Staging {
   char* p = nullptr;
@@ -633,6 +644,27 @@ struct Staging {
   Staging(const Staging&) = delete;
   Staging& operator=(const Staging&) = delete;
 };
+
+}  // namespace
+
+LiveHandle::LiveHandle() {
+  std::lock_guard<std::mutex> lock(g_staging_mu);
+  ++g_handles;
+}
+
+LiveHandle::~LiveHandle() {
+  std::vector<char*> back;
+  {
+    std::lock_guard<std::mutex> lock(g_staging_mu);
+    if (--g_handles == 0 && g_staging.size() > 1) {
+      back.assign(g_staging.begin() + 1, g_staging.end());
+      g_staging.resize(1);
+    }
+  }
+  for (char* q : back) cudaFreeHost(q);
+}
+
+namespace {
 
 // Wait for the handle's stream, take over its error flags, and copy out what is wanted of the
 // state (null: not).  After a non-finite or timed-out step the state is copied all the same;
