@@ -19,7 +19,7 @@
 // Bound by the FP32 pipe at n = 8192 (half of its rate: few warps, the split of the positions
 // in every CTA) and by the launch and one chunk's latency below ~2000.  Measured back to back on
 // GB300, us per call, the previous two clears and two launches against this kernel: n = 64:
-// 17 -> 8.3, 1000: 21 -> 10.3, 3000: 32 -> 16.3, 5000: 46 -> 27, 8192: 77 -> 55.
+// 17 -> 8.3, 1000: 21 -> 8.3, 3000: 32 -> 14.4, 5000: 46 -> 24.6, 8192: 77 -> 52.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -47,10 +47,13 @@ struct ForcesArgs {
   float w[IONTRAP_MAX_SPECIES];
 };
 
-// I ions per lane: 1, or 2 packed.
-template <int I, bool UNITW>
-__global__ void __launch_bounds__(32 * kMaxChunks) k_forces_cluster(const __grid_constant__ ForcesArgs A) {
-  constexpr int kBlockIons = 32 * I;
+// I ions per lane: 1, or 2 packed.  M: CTAs of eight warps that the registers leave room for, at
+// least.  Without that bound the compiler took 158 for the pair loop written in stages of 16 j and
+// two CTAs of five warps shared an SM (n = 5000: 28.5 us a call, 24.6 with M = 1 and 95 registers);
+// 64 registers (M = 4) take stages of 4 j.
+template <int I, bool UNITW, int M>
+__global__ void __launch_bounds__(32 * kMaxChunks, M) k_forces_cluster(const __grid_constant__ ForcesArgs A) {
+  constexpr int kBlockIons = 32 * I, kStage = M == 1 ? 16 : 4;
   __shared__ __align__(16) float4 sh[kMaxChunks][kSeg], sl[kMaxChunks][kSeg];
   __shared__ float s_sum[kMaxChunks][3][kBlockIons];   // chunk sums; row 0 then the CTA's Kahan sum
   __shared__ float s_comp[3][kBlockIons];              // and compensation
@@ -109,9 +112,9 @@ __global__ void __launch_bounds__(32 * kMaxChunks) k_forces_cluster(const __grid
       for (int d = 0; d < 3; ++d) acc[0][d].x = a1[0][d];
     } else {
       if (diag)
-        segment_f32x2<I, true, UNITW>(sh[warp], sl[warp], jn, jc, nxh, nxl, ii, acc);
+        segment_f32x2<I, true, UNITW, kStage>(sh[warp], sl[warp], jn, jc, nxh, nxl, ii, acc);
       else
-        segment_f32x2<I, false, UNITW>(sh[warp], sl[warp], jn, jc, nxh, nxl, ii, acc);
+        segment_f32x2<I, false, UNITW, kStage>(sh[warp], sl[warp], jn, jc, nxh, nxl, ii, acc);
     }
 #pragma unroll
     for (int k = 0; k < I; ++k)
@@ -181,8 +184,11 @@ extern "C" int iontrap_forces_noalloc(const iontrap_species* species, int n_spec
   }
   cudaLaunchConfig_t cfg{};
   // one ion per lane while the chip is short of warps (us per call, 1 / 2 ions per lane:
-  // n = 1000: 10.3 / 12.4, 3000: 16.3 / 16.5, 4097: 24.3 / 19.6, 8192: 62 / 55)
-  const int I = n <= 3200 ? 1 : 2;
+  // n = 2600: 12.3 / 14.4, 3201: 16.4 / 14.4, 4097: 22.6 / 18.5, 8192: 60 / 54); and from seven
+  // warps a CTA on four CTAs per SM rather than three (M = 1 / 4: n = 5000: 24.6 / 26.7, 6000:
+  // 32.8 / 32.8, 7000: 45.9 / 39.2, 8192: 53.8 / 52.1; with a doubly charged species 7000: 48.7 / 41.1)
+  const int I = n <= 2800 ? 1 : 2;
+  const bool four = A.jsplit > 6 * kSeg;
   cfg.gridDim = dim3((unsigned)((n + 32 * I - 1) / (32 * I)), nsplit);
   cfg.blockDim = dim3(32u * (unsigned)((A.jsplit + kSeg - 1) / kSeg));
   cfg.stream = static_cast<cudaStream_t>(cuda_stream);
@@ -194,7 +200,8 @@ extern "C" int iontrap_forces_noalloc(const iontrap_species* species, int n_spec
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   const cudaError_t e = cudaLaunchKernelEx(
-      &cfg, I == 1 ? (unitw ? k_forces_cluster<1, true> : k_forces_cluster<1, false>)
-                   : (unitw ? k_forces_cluster<2, true> : k_forces_cluster<2, false>), A);
+      &cfg, I == 1 ? (unitw ? k_forces_cluster<1, true, 1> : k_forces_cluster<1, false, 1>)
+            : four ? (unitw ? k_forces_cluster<2, true, 4> : k_forces_cluster<2, false, 4>)
+                   : (unitw ? k_forces_cluster<2, true, 1> : k_forces_cluster<2, false, 1>), A);
   return e == cudaSuccess ? IONTRAP_OK : IONTRAP_ECUDA;
 }

@@ -390,12 +390,11 @@ __device__ __forceinline__ void group_f32x2(const float4* __restrict__ sh, const
     }
 }
 
-template <int I, bool DIAG, bool UNITW = false>
+template <int I, bool DIAG, bool UNITW = false, int V = I == 2 ? 16 : 3>
 __device__ __forceinline__ void segment_f32x2(const float4* __restrict__ sh, const float4* __restrict__ sl, int jn,
                                               long long jbase, const float2 (&nxh)[I / 2][3],
                                               const float2 (&nxl)[I / 2][3], const long long (&ii)[I],
                                               float2 (&acc)[I / 2][3]) {
-  constexpr int V = I == 2 ? 16 : 3;
   int j = 0;
 #pragma unroll 1
   for (; j + V <= jn; j += V) group_f32x2<I, V, DIAG, UNITW>(sh, sl, j, jbase, nxh, nxl, ii, acc);

@@ -8,7 +8,7 @@ import iongen
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n", [1, 2, 31, 33, 64, 127, 128, 129, 300, 513, 700, 896, 1025, 3200, 3201, 4099, 8191, 8192])
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 64, 127, 128, 129, 300, 513, 700, 896, 1025, 2800, 2801, 3200, 3201, 4099, 6144, 6145, 7169, 8191, 8192])
 @pytest.mark.parametrize("unit", [True, False])
 def test_noalloc_forces_are_the_last_cta_forces(n, unit):
     import torch
