@@ -453,20 +453,31 @@ int iontrap_forces_noalloc(const iontrap_species *species, int n_species, const 
 
 /* Test hook of the failure detection (no counterpart in the paper).  Every wait of the persistent forms 4 and 5
  * -- a CTA's poller waiting for the other CTAs' arrivals on a step or group counter, a
- * CTA waiting for its bulk copies -- gives up after a time limit, sets the handle's
+ * CTA waiting for its bulk copies, a cluster's CTA waiting for the others' positions -- gives up
+ * after a time limit, sets the handle's
  * timeout flag and ends the launch, which the host reads as IONTRAP_ETIMEOUT.  This hook
  * makes that happen on purpose, with no fault and no unbounded wait: the persistent
  * launches of the handle that follow use a limit of wait_limit_ns (0 restores the default,
  * 2 s), and when cta >= 0, CTA number cta withholds its arrival on the grid-wide step
  * counter at step `step` (counted from 0 within each launch) -- a counter value nothing
- * will reach -- so that every other CTA's wait for the next step expires after the
+ * will reach -- or, where steps run on one cluster, its positions after that step (none are sent
+ * after a launch's last), so that every other CTA's wait for the next step expires after the
  * limit.  The launch then stops, the handle's status becomes IONTRAP_ETIMEOUT (sticky)
  * and its step index is not advanced; in form 5 the FP64 state is the one the launch
  * started from, in form 4 it may hold some of the launch's steps.  cta < 0 turns the stall
- * off.  Synchronous (waits for queued work).  EINVAL when the handle is not in form 4 or
- * 5, when its launch has a single CTA (form 5 up to 170 ions: no cross-CTA wait), or when
+ * off; a form 5 handle with a limit and no stall steps on the grid with its counter, whose bits the
+ * other kernels of the form are compared with.  Synchronous (waits for queued work).  EINVAL when
+ * the handle is not in form 4 or
+ * 5, when its launch has a single CTA (no cross-CTA wait), or when
  * cta is not below the launch's CTA count. */
 int iontrap_test_stall(iontrap_t *h, int64_t wait_limit_ns, int32_t cta, int64_t step);
+
+/* Test hook: the kernel (IONTRAP_KERNEL_*) and the CTAs that the steps of a handle in form 5 run
+ * on, under the settings of iontrap_test_stall.  EINVAL when the handle is in another form. */
+#define IONTRAP_KERNEL_GRID 0    /* the grid, a counter and bulk copies (or one CTA) */
+#define IONTRAP_KERNEL_TAGGED 1  /* the grid, tagged positions */
+#define IONTRAP_KERNEL_CLUSTER 2 /* one thread-block cluster */
+int iontrap_test_step_kernel(const iontrap_t *h, int32_t *kernel, int32_t *ctas);
 
 /* Profiling hook: run ONE step with per-CTA phase timestamps (%globaltimer, ns) and copy
  * them to marks[cap] (EINVAL in the grid-persistent form 4; in the row-persistent form 5

@@ -38,11 +38,12 @@ constexpr int kRpcOwners = 128, kRpcNoise = 64, kRpcPairs = 448;  // threads of 
 constexpr int kRpcThreads = kRpcOwners + kRpcNoise + kRpcPairs;   // 20 warps: 5 per sub-partition
 constexpr int kRpcNoiseWarp = 7;                                  // and the one before it: the sub-partitions of owner
                                                                   // warps 3 and 2, which own ions last
-constexpr int kRpcMaxRc = 40;                                     // ions per CTA: 3 x 40 owner threads
+constexpr int kRpcMaxRc = 40;                                     // entries per CTA: 3 x 40 owner threads
 constexpr int kRpcMaxN = 432;                                     // measured: see rpc_ctas
 constexpr int kRpcGroups = 8;                                     // rounds are handed over in at most this many groups
 // named barriers: 1 .. kRpcGroups the groups of rounds, then
-constexpr int kRpcBarNoise = 9, kRpcBarLaser = 10;
+constexpr int kRpcBarStep = 9, kRpcBarLaser = 10;
+constexpr unsigned long long kRpcSettleNs = 20000;                // stores in flight land in ~1 us
 
 struct RpcArgs {
   long long K;  // steps in this launch
@@ -71,6 +72,16 @@ __device__ __forceinline__ void bar_sync(int id, int threads) {
 }
 __device__ __forceinline__ void bar_arrive(int id, int threads) {
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// Wait for the positions, giving up after limit ns or when another warp of the CTA has (*given).
+__device__ __forceinline__ bool rpc_wait(uint64_t* bar, uint32_t parity, unsigned long long limit,
+                                         const volatile int* given) {
+  if (mbar_try_wait(bar, parity)) return true;
+  const unsigned long long t0 = globaltimer_ns();
+  while (!mbar_try_wait(bar, parity))
+    if (*given || globaltimer_ns() - t0 > limit) return false;
+  return true;
 }
 
 // Part sums are kept [part][kRpcOwners] by owner thread: constant offsets for the merge.
@@ -109,7 +120,7 @@ __global__ void __launch_bounds__(kRpcThreads, 1) k_step_f32_rpc(const __grid_co
   // [2][species][3]
   extern __shared__ __align__(16) float4 s_dyn[];
   __shared__ __align__(8) uint64_t bar[2];  // positions of a buffer complete
-  __shared__ volatile int s_bad;            // a wait of this CTA gave up
+  __shared__ volatile int s_bad[2];         // a wait of this CTA gave up in an even, an odd step
   cg::cluster_group cluster = cg::this_cluster();
   const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int tid = threadIdx.x;
@@ -134,9 +145,10 @@ __global__ void __launch_bounds__(kRpcThreads, 1) k_step_f32_rpc(const __grid_co
   const TrapDev& tp = A.trap;
   const long long ns0 = *A.step;
   const bool rf = !(tp.flags & (IONTRAP_RF_OFF | IONTRAP_TRAP_OFF | IONTRAP_PSEUDO));
+  const unsigned long long lim = A.wait_ns ? A.wait_ns : kWaitLimitNs;
 
   if (tid == 0) {
-    s_bad = 0;
+    s_bad[0] = s_bad[1] = 0;
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
     for (int b = 0; b < 2; ++b) mbar_arrive_expect_tx(&bar[b], step_bytes);
@@ -190,6 +202,14 @@ __global__ void __launch_bounds__(kRpcThreads, 1) k_step_f32_rpc(const __grid_co
   const int rounds = (NPe + G - 1) / G;
   const int per = (rounds + kRpcGroups - 1) / kRpcGroups, groups = (rounds + per - 1) / per;
 
+  // A wait that gives up ends the launch for the whole CTA at one step: the warp sets the step's
+  // s_bad before it passes on its groups, so the value is settled when the owners have merged and
+  // when the 20 warps have met at kRpcBarStep, after which they leave by it.  No pair warp is in the
+  // next step before that barrier, and that step has a flag of its own; the step after it, which
+  // has this one again, begins when every warp has read it.  A launch's last step ends without the
+  // barrier: nothing waits after it.  (That the pair warps come to the barrier costs nothing: the
+  // positions that they wait for next are in flight for longer.  64 ions, 200 steps and the state:
+  // 267 us with 6 warps at the barrier, 267 with 20.)
   if (warp > kRpcNoiseWarp || (warp >= kRpcOwners / 32 && warp < kRpcNoiseWarp - 1)) {  // -------- pair warps
     const int pt = tid - kRpcOwners - (warp > kRpcNoiseWarp ? kRpcNoise : 0);
     const int first = pt / Rg, s = pt - first * Rg;
@@ -198,11 +218,12 @@ __global__ void __launch_bounds__(kRpcThreads, 1) k_step_f32_rpc(const __grid_co
     for (int t = 0; t < K; ++t) {
       const int cur = t & 1;
       if (t > 0) {
-        const bool ok = mbar_wait_bounded(&bar[cur], (uint32_t)(((t - 1) >> 1) & 1), kWaitLimitNs);
-        if (__any_sync(0xffffffffu, !ok)) {  // flag, let the owners go, give up
-          s_bad = 1;
+        const bool ok = rpc_wait(&bar[cur], (uint32_t)(((t - 1) >> 1) & 1), lim, &s_bad[cur]);
+        if (__any_sync(0xffffffffu, !ok)) {  // give up; the owners and the other warps follow
+          s_bad[cur] = 1;
           __threadfence_block();
           for (int g = 0; g < groups; ++g) bar_arrive(1 + g, kRpcOwners + kRpcPairs);
+          if (t + 1 < K) bar_sync(kRpcBarStep, kRpcThreads);
           break;
         }
         // armed again for the positions two steps on: their senders wait for this CTA's own
@@ -210,13 +231,16 @@ __global__ void __launch_bounds__(kRpcThreads, 1) k_step_f32_rpc(const __grid_co
         if (pt == 0) mbar_arrive_expect_tx(&bar[cur], step_bytes);
       }
       rpc_parts<UNITW>(buf + cur * blen, wz, ps + s, Rg4, JP, NPe, G, per, groups, first, i, on);
+      if (t + 1 == K) break;
+      bar_sync(kRpcBarStep, kRpcThreads);
+      if (s_bad[cur]) break;
     }
   } else if (tid >= kRpcOwners) {  // -------------------------------------------- noise warps
     for (int t = 0; t + 1 < K; ++t) {
       if (warp == kRpcNoiseWarp) springs(t + 1);
       if (noisy) draw(t + 1);
-      bar_sync(kRpcBarNoise, kRpcOwners + kRpcNoise);
-      if (s_bad) break;
+      bar_sync(kRpcBarStep, kRpcThreads);
+      if (s_bad[t & 1]) break;
     }
   } else {  // ------------------------------------------------------------------- owner warps
     // thread k < 3 Rg4 integrates component k / Rg4 of ion r0 + k % Rg4 (a padding entry
@@ -258,6 +282,8 @@ __global__ void __launch_bounds__(kRpcThreads, 1) k_step_f32_rpc(const __grid_co
       rdst[k] = map_rank(smem_u32(buf + (owns ? rpc_at(ie & ~3, oc) : 0)), r);
       rbar[k] = map_rank(smem_u32(&bar[0]), r);
     }
+    // the step after which a CTA that the failure test stalls keeps its positions to itself
+    const int stall_t = A.stall_on && rank == A.stall_cta && A.stall_step < K ? (int)A.stall_step : -1;
     ext_of(0);
     for (int t = 0; t < K; ++t) {
       const int cur = t & 1;
@@ -296,7 +322,7 @@ __global__ void __launch_bounds__(kRpcThreads, 1) k_step_f32_rpc(const __grid_co
 #pragma unroll 1
         for (; p < p1; ++p, q += kRpcOwners) add(q[0]);
       }
-      const bool bad = s_bad != 0;
+      const bool bad = s_bad[cur] != 0;
       float h = 1e30f, l = 0.0f;
       if (own && !bad) {
         const double Sd = widen(cu) - widen(su);
@@ -322,7 +348,7 @@ __global__ void __launch_bounds__(kRpcThreads, 1) k_step_f32_rpc(const __grid_co
         xf = xn;
       }
       if (t + 1 == K) break;
-      if (owns && !bad) {
+      if (owns && !bad && t != stall_t) {
         // four consecutive threads hold four consecutive ions: each collects the four and
         // stores them to every fourth CTA
         const int base = tid & 28;
@@ -337,13 +363,18 @@ __global__ void __launch_bounds__(kRpcThreads, 1) k_step_f32_rpc(const __grid_co
             st_async4(rdst[k] + to + 48u, l4, rbar[k] + tb);
           }
       }
-      bar_sync(kRpcBarNoise, kRpcOwners + kRpcNoise);  // the next step's normals are there
+      bar_sync(kRpcBarStep, kRpcThreads);  // the next step's normals are there
       if (bad) break;
       ext_of(t + 1);
     }
-    if (tid == 0 && s_bad) atomicOr(A.err, ERR_TIMEOUT);
+    if (tid == 0 && (s_bad[0] | s_bad[1])) atomicOr(A.err, ERR_TIMEOUT);
   }
-  cluster.sync();  // every store has landed or its CTA has given up: nobody leaves before
+  cluster.sync();  // every store has been sent, and has landed in the CTAs that did not give up
+  if (s_bad[0] | s_bad[1]) {  // others' stores may be in flight to this one
+    const unsigned long long t0 = globaltimer_ns();
+    while (globaltimer_ns() - t0 < kRpcSettleNs) {
+    }
+  }
   if (rank == 0 && tid == 0 && !(*(volatile int*)A.err & ERR_TIMEOUT)) *A.step = ns0 + P.K;
 }
 

@@ -746,20 +746,32 @@ int alloc_scratch(iontrap* h) {
   return IONTRAP_OK;
 }
 
+// The kernel of a row-persistent launch, and its CTAs: steps of a small simulation run on one
+// cluster, those of the next sizes on the grid with tagged positions (the same bits all three).
+// Force evaluations take the grid with its counter, as do steps with a wait limit of their own and
+// no stall (iontrap_test_stall), for comparisons; traced launches, marked per CTA of the grid, keep
+// off the cluster.
+int rp_kernel_of(const iontrap* h, const StepArgs& a, int* ctas) {
+  *ctas = h->rp.G;
+  if (a.mode != MODE_STEP || (a.wait_ns && !a.stall_on)) return IONTRAP_KERNEL_GRID;
+  const int C = a.trace ? 0 : rpc_ctas(h->n, h->rp.JP);
+  if (tag_takes(h->n, h->rp.W, h->rp.R, h->rp.JP, h->rp.G, h->sms, C > 0))
+    return a.wait_ns || a.stall_on ? IONTRAP_KERNEL_GRID : IONTRAP_KERNEL_TAGGED;
+  if (C == 0) return IONTRAP_KERNEL_GRID;
+  *ctas = C;
+  return IONTRAP_KERNEL_CLUSTER;
+}
+
 // One row-persistent launch of K steps on the handle's buffers.
 cudaError_t launch_rp_of(iontrap* h, const StepArgs& a, long long K, cudaStream_t st) {
-  // steps of a small simulation run on one cluster, those of the next sizes on the grid with
-  // tagged positions (the same bits all three); force evaluations and launches of the failure
-  // test, which look at the grid's counter, do not, and traced launches, marked per CTA of the
-  // grid, keep off the cluster
-  if (a.mode == MODE_STEP && !a.stall_on && !a.wait_ns) {
-    const int C = a.trace ? 0 : rpc_ctas(h->n, h->rp.JP);
-    if (tag_takes(h->n, h->rp.W, h->rp.R, h->rp.JP, h->rp.G, h->sms, C > 0))
+  int ctas;
+  switch (rp_kernel_of(h, a, &ctas)) {
+    case IONTRAP_KERNEL_CLUSTER: return launch_rpc(a, h->nspecies, ctas, h->rp.JP, K, st);
+    case IONTRAP_KERNEL_TAGGED:
       return launch_tag(a, h->d_gsync, h->d_gsync + kGpSyncBytes / sizeof(unsigned), h->rp.R, h->rp.JP, h->rp.I,
                         h->rp.G, K, st);
-    if (C > 0) return launch_rpc(a, h->nspecies, C, h->rp.JP, K, st);
+    default: return launch_rp(a, h->d_gsync, h->rp.W, h->rp.R, h->rp.NP, h->rp.JP, h->rp.I, h->rp.G, K, st);
   }
-  return launch_rp(a, h->d_gsync, h->rp.W, h->rp.R, h->rp.NP, h->rp.JP, h->rp.I, h->rp.G, K, st);
 }
 
 // Launch one step kernel with programmatic dependent launch, so that consecutive steps
@@ -1463,16 +1475,33 @@ int iontrap_restore(iontrap_t* h, const double* x, const double* v, const double
 
 int iontrap_test_stall(iontrap_t* h, int64_t wait_limit_ns, int32_t cta, int64_t step) {
   if (!h || wait_limit_ns < 0 || step < 0 || (h->fused != 4 && h->fused != 5)) return IONTRAP_EINVAL;
-  const int ctas = h->fused == 4 ? h->gp.G : h->rp.G;
+  StepArgs a = h->args;
+  a.mode = MODE_STEP;
+  a.wait_ns = (unsigned long long)wait_limit_ns;
+  a.stall_on = cta >= 0 ? 1 : 0;
+  a.stall_cta = cta >= 0 ? cta : 0;
+  a.stall_step = step;
+  int ctas = h->gp.G;
+  if (h->fused == 5) rp_kernel_of(h, a, &ctas);
   if (cta >= ctas || ctas < 2) return IONTRAP_EINVAL;  // one CTA waits on no other
   if (h->status) return h->status;
   DeviceGuard g(h->device);
   const cudaError_t e = cudaStreamSynchronize(h->stream);  // launches already queued keep their settings
   if (e != cudaSuccess) return cuda_status(h, e);
-  h->args.wait_ns = (unsigned long long)wait_limit_ns;
-  h->args.stall_on = cta >= 0 ? 1 : 0;
-  h->args.stall_cta = cta >= 0 ? cta : 0;
-  h->args.stall_step = step;
+  h->args.wait_ns = a.wait_ns;
+  h->args.stall_on = a.stall_on;
+  h->args.stall_cta = a.stall_cta;
+  h->args.stall_step = a.stall_step;
+  return IONTRAP_OK;
+}
+
+int iontrap_test_step_kernel(const iontrap_t* h, int32_t* kernel, int32_t* ctas) {
+  if (!h || !kernel || !ctas || h->fused != 5) return IONTRAP_EINVAL;
+  StepArgs a = h->args;
+  a.mode = MODE_STEP;
+  int c;
+  *kernel = rp_kernel_of(h, a, &c);
+  *ctas = c;
   return IONTRAP_OK;
 }
 

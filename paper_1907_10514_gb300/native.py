@@ -39,6 +39,10 @@ IONTRAP_PREC_FP32 = 0
 IONTRAP_PREC_FP64 = 1
 IONTRAP_TUNE_BATCHED = 2
 
+IONTRAP_KERNEL_GRID = 0
+IONTRAP_KERNEL_TAGGED = 1
+IONTRAP_KERNEL_CLUSTER = 2
+
 IONTRAP_MAX_SPECIES = 16
 
 
@@ -135,6 +139,7 @@ SIGNATURES = {
     "iontrap_server_destroy": (None, [_vp]),
     "iontrap_trace_step": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_ulonglong), ctypes.c_int64, _i64p, _i64p]),
     "iontrap_test_stall": (ctypes.c_int, [_vp, ctypes.c_int64, ctypes.c_int32, ctypes.c_int64]),
+    "iontrap_test_step_kernel": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32)]),
     "iontrap_alu_probe": (ctypes.c_int, [ctypes.c_longlong, ctypes.c_longlong, _dp, _dp]),
 }
 
@@ -307,6 +312,13 @@ def iontrap_state(h, n: int, x_out: Optional[np.ndarray] = None, v_out: Optional
 
 def iontrap_test_stall(h, wait_limit_ns: int, cta: int, step: int) -> None:
     _check(_lib.iontrap_test_stall(h, int(wait_limit_ns), int(cta), int(step)), "iontrap_test_stall")
+
+
+def iontrap_test_step_kernel(h):
+    """(kernel, CTAs) of a form 5 handle's steps: IONTRAP_KERNEL_GRID, _TAGGED or _CLUSTER."""
+    kernel, ctas = ctypes.c_int32(-1), ctypes.c_int32(0)
+    _check(_lib.iontrap_test_step_kernel(h, ctypes.byref(kernel), ctypes.byref(ctas)), "iontrap_test_step_kernel")
+    return kernel.value, ctas.value
 
 
 def iontrap_forces(h, n: int) -> np.ndarray:
