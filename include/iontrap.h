@@ -229,8 +229,9 @@ int iontrap_sync(iontrap_t *h);
 /* Synchronise, then copy out the state: x[3n], v[3n] (either may be NULL), the step
  * index *step and time *t = step dt (either may be NULL).  After a device-side failure
  * (IONTRAP_ENONFINITE, IONTRAP_ETIMEOUT) the state is still copied out -- for a timeout in
- * the row-persistent form it is the state the failed launch started from -- and the
- * sticky status is returned. */
+ * the row-persistent form it is the state the failed launch started from, unless the wait
+ * that gave up was for or after the launch's last step, when some ions may have taken it
+ * -- and the sticky status is returned. */
 int iontrap_state(iontrap_t *h, double *x, double *v, int64_t *step, double *t);
 
 /* Synchronise, then write the Coulomb acceleration k_e e^2 z_i/M_i sum_j z_j d_ij/r_ij^3
@@ -453,18 +454,19 @@ int iontrap_forces_noalloc(const iontrap_species *species, int n_species, const 
 
 /* Test hook of the failure detection (no counterpart in the paper).  Every wait of the persistent forms 4 and 5
  * -- a CTA's poller waiting for the other CTAs' arrivals on a step or group counter, a
- * CTA waiting for its bulk copies, a cluster's CTA waiting for the others' positions -- gives up
- * after a time limit, sets the handle's
+ * CTA waiting for its bulk copies, a CTA waiting for the others' positions (tagged on the grid,
+ * counted in a cluster) -- gives up after a time limit, sets the handle's
  * timeout flag and ends the launch, which the host reads as IONTRAP_ETIMEOUT.  This hook
  * makes that happen on purpose, with no fault and no unbounded wait: the persistent
  * launches of the handle that follow use a limit of wait_limit_ns (0 restores the default,
  * 2 s), and when cta >= 0, CTA number cta withholds its arrival on the grid-wide step
  * counter at step `step` (counted from 0 within each launch) -- a counter value nothing
- * will reach -- or, where steps run on one cluster, its positions after that step (none are sent
- * after a launch's last), so that every other CTA's wait for the next step expires after the
- * limit.  The launch then stops, the handle's status becomes IONTRAP_ETIMEOUT (sticky)
+ * will reach -- or, where positions are tagged or counted, its positions after that step (in a
+ * cluster nothing is sent after a launch's last; on the grid its arrival there), so that every
+ * other CTA's wait for the next step expires after the limit.  The launch then stops, the handle's status becomes IONTRAP_ETIMEOUT (sticky)
  * and its step index is not advanced; in form 5 the FP64 state is the one the launch
- * started from, in form 4 it may hold some of the launch's steps.  cta < 0 turns the stall
+ * started from (a stall at the launch's last step, whose positions nobody needs, leaves the
+ * state after it), in form 4 it may hold some of the launch's steps.  cta < 0 turns the stall
  * off; a form 5 handle with a limit and no stall steps on the grid with its counter, whose bits the
  * other kernels of the form are compared with.  Synchronous (waits for queued work).  EINVAL when
  * the handle is not in form 4 or

@@ -755,8 +755,7 @@ int rp_kernel_of(const iontrap* h, const StepArgs& a, int* ctas) {
   *ctas = h->rp.G;
   if (a.mode != MODE_STEP || (a.wait_ns && !a.stall_on)) return IONTRAP_KERNEL_GRID;
   const int C = a.trace ? 0 : rpc_ctas(h->n, h->rp.JP);
-  if (tag_takes(h->n, h->rp.W, h->rp.R, h->rp.JP, h->rp.G, h->sms, C > 0))
-    return a.wait_ns || a.stall_on ? IONTRAP_KERNEL_GRID : IONTRAP_KERNEL_TAGGED;
+  if (tag_takes(h->n, h->rp.W, h->rp.R, h->rp.JP, h->rp.G, h->sms, C > 0)) return IONTRAP_KERNEL_TAGGED;
   if (C == 0) return IONTRAP_KERNEL_GRID;
   *ctas = C;
   return IONTRAP_KERNEL_CLUSTER;

@@ -698,8 +698,9 @@ __global__ void __launch_bounds__(32 * W, 1) k_step_f32_rp(const __grid_constant
   }
 
   // once every CTA has counted its last step: clear the counter, advance the step index.
-  // A launch that gave up on a wait leaves both alone: its FP64 state is still the one it
-  // started from, and the handle's sticky timeout status retires the counter with it.
+  // A launch that gave up on a wait leaves both alone, and the handle's sticky timeout status
+  // retires the counter with it.  Its FP64 state is still the one it started from, unless the
+  // wait was for or after the launch's last step: CTAs that finished that have written theirs.
   if (blockIdx.x == 0 && tid == poller) {
     if (solo || poll_wait<true>(ctr_step, G * (unsigned)P.K, A.err, lim)) {
       *ctr_step = 0u;

@@ -80,12 +80,13 @@ __device__ __forceinline__ void bar_arrive(int id, int threads) {
 }
 
 // Given up on a wait: the limit has passed, or another thread has given up.
-static __device__ __noinline__ bool tag_late(unsigned long long& t0, int* err) {
-  if (*(volatile int*)err & ERR_TIMEOUT) return true;
+__device__ __forceinline__ unsigned long long tag_limit(const StepArgs& A) { return A.wait_ns ? A.wait_ns : kWaitLimitNs; }
+static __device__ __noinline__ bool tag_late(unsigned long long& t0, const StepArgs& A) {
+  if (*(volatile int*)A.err & ERR_TIMEOUT) return true;
   const unsigned long long now = globaltimer_ns();
   if (!t0) t0 = now;
-  if (now - t0 <= kWaitLimitNs) return false;
-  atomicOr(err, ERR_TIMEOUT);
+  if (now - t0 <= tag_limit(A)) return false;
+  atomicOr(A.err, ERR_TIMEOUT);
   return true;
 }
 
@@ -94,7 +95,7 @@ static __device__ __noinline__ bool tag_late(unsigned long long& t0, int* err) {
 // reads are in flight.  False if the wait was given up.
 template <int U>
 static __device__ __forceinline__ bool tag_fetch(const uint4* src, int items, int first, int stride, unsigned tag,
-                                                 float* dst, int JP, unsigned magic, int* err) {
+                                                 float* dst, int JP, unsigned magic, const StepArgs& A) {
   unsigned long long late = 0;
   unsigned it = 0;
   for (int m0 = first; m0 < items; m0 += U * stride) {
@@ -115,7 +116,7 @@ static __device__ __forceinline__ bool tag_fetch(const uint4* src, int items, in
           d[0] = __uint_as_float(a[u].x), d[JP] = __uint_as_float(a[u].y), d[2 * JP] = __uint_as_float(a[u].z);
         }
       if (!pend) break;
-      if ((++it & 63u) == 0 && tag_late(late, err)) return false;
+      if ((++it & 63u) == 0 && tag_late(late, A)) return false;
     }
   }
   return true;
@@ -140,6 +141,8 @@ __global__ void __launch_bounds__(kTagThreads, 1) k_step_f32_tag(const __grid_co
   const unsigned tag0 = *(volatile unsigned*)P.tags;
   uint4* const ent = reinterpret_cast<uint4*>(reinterpret_cast<char*>(P.tags) + kTagHeader);
   const bool rf = !(tp.flags & (IONTRAP_RF_OFF | IONTRAP_TRAP_OFF | IONTRAP_PSEUDO));
+  // the step after which a CTA that the failure test stalls publishes nothing
+  const int stall_t = A.stall_on && (int)blockIdx.x == A.stall_cta && A.stall_step < K ? (int)A.stall_step : -1;
   for (int k = tid; k < K; k += kTagThreads) scos[k] = rf ? cos(tp.Omega * ((double)(ns0 + k + 1) * tp.dt)) : 0.0;
 
   // pair work: ion slot (slots slot and slot + RT with two ions per thread) and j-part
@@ -225,7 +228,7 @@ __global__ void __launch_bounds__(kTagThreads, 1) k_step_f32_tag(const __grid_co
       const int PT = kTagThreads - ow, half = tid & 1;
       float* const base = sall + 3 * half * JP;
       bar_sync(kTagBarPublished, kTagThreads);
-      bad = !tag_fetch<U>(src, 2 * n, tid - ow, PT, tag, base, JP, P.magic, A.err);
+      bad = !tag_fetch<U>(src, 2 * n, tid - ow, PT, tag, base, JP, P.magic, A);
     }
     if (__syncthreads_or(bad)) {
       bad = true;
@@ -339,7 +342,7 @@ __global__ void __launch_bounds__(kTagThreads, 1) k_step_f32_tag(const __grid_co
       }
       if (t + 1 < K) {
         bar_sync(kTagBarOwners, ow);
-        if (tid < 2 * Rg) {  // publish: half hf of ion q
+        if (tid < 2 * Rg && t != stall_t) {  // publish: half hf of ion q
           const int q = tid >> 1, hf = tid & 1;
           const unsigned tag = tag0 + (unsigned)t + 1u;
           const float* s = sself + 3 * hf * R + q;
@@ -353,12 +356,13 @@ __global__ void __launch_bounds__(kTagThreads, 1) k_step_f32_tag(const __grid_co
   }
 
   // Once every CTA has read its last positions: clear the counter, advance the step index
-  // and the tag.  A launch that gave up on a wait leaves all three alone: its FP64 state is
-  // still the one it started from, and the handle's sticky timeout status retires them.
+  // and the tag.  A launch that gave up on a wait leaves all three alone, and the handle's sticky
+  // timeout status retires them.  Its FP64 state is still the one it started from, unless the wait
+  // was for the launch's last step: CTAs that received its positions have written theirs.
   __syncthreads();
   if (tid == 0) {
-    if (!bad) arrive_release(P.sync);
-    if (blockIdx.x == 0 && poll_wait<true>(P.sync, gridDim.x, A.err, kWaitLimitNs)) {
+    if (!bad && stall_t != K - 1) arrive_release(P.sync);
+    if (blockIdx.x == 0 && poll_wait<true>(P.sync, gridDim.x, A.err, tag_limit(A))) {
       *P.sync = 0u;
       *P.tags = tag0 + (unsigned)(K - 1);
       *A.step = ns0 + K;

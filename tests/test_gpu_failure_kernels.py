@@ -28,8 +28,10 @@ def _handle(it, n, laser):
     return s
 
 
-# default handles: clusters of 4, 8 and 16 CTAs
-CASES = [(13, "CLUSTER", 4), (64, "CLUSTER", 8), (150, "CLUSTER", 16)]
+# default handles: clusters of 4, 8 and 16 CTAs; tagged positions with 8, 16 and 24 reads in flight
+# and a last CTA of fewer ions
+CASES = [(13, "CLUSTER", 4), (64, "CLUSTER", 8), (150, "CLUSTER", 16),
+         (300, "TAGGED", 150), (1000, "TAGGED", 143), (2047, "TAGGED", 147)]
 
 
 @pytest.mark.parametrize("n,kernel,ctas", CASES)
@@ -74,3 +76,18 @@ def test_a_limit_that_is_not_reached_changes_nothing(n, kernel, ctas):
             got.append(s.checkpoint())
     for u, w in zip(*got):
         assert np.array_equal(u, w)
+
+
+def test_a_withheld_last_arrival_is_a_timeout_too():
+    """The grid counts its CTAs once after a launch's last step."""
+    import paper_1907_10514_gb300 as it
+    n = 300
+    with _handle(it, n, False) as s:
+        it.iontrap_test_stall(s.handle, LIMIT_NS, 7, K - 1)
+        assert it.iontrap_test_step_kernel(s.handle)[0] == it.IONTRAP_KERNEL_TAGGED
+        s.step(K)
+        with pytest.raises(it.IonTrapError) as e:
+            s.sync()
+        assert e.value.code == it.IONTRAP_ETIMEOUT
+        x, v, step, _ = it.iontrap_state(s.handle, n, accept=(it.IONTRAP_ETIMEOUT,))
+        assert step == 0
