@@ -466,7 +466,10 @@ int iontrap_forces_noalloc(const iontrap_species *species, int n_species, const 
  * other CTA's wait for the next step expires after the limit.  The launch then stops, the handle's status becomes IONTRAP_ETIMEOUT (sticky)
  * and its step index is not advanced; in form 5 the FP64 state is the one the launch
  * started from (a stall at the launch's last step, whose positions nobody needs, leaves the
- * state after it), in form 4 it may hold some of the launch's steps.  cta < 0 turns the stall
+ * state after it), in form 4 it may hold some of the launch's steps.  iontrap_minimize in form 5
+ * above 432 ions, whose iterations meet at barriers of the grid, is stalled at barrier `step` of
+ * its launches (three per iteration; up to 432 ions a cluster's hardware barriers have no wait to
+ * bound) and returns IONTRAP_ETIMEOUT, with positions that may hold some moves.  cta < 0 turns the stall
  * off; a form 5 handle with a limit and no stall steps on the grid with its counter, whose bits the
  * other kernels of the form are compared with.  Synchronous (waits for queued work).  EINVAL when
  * the handle is not in form 4 or

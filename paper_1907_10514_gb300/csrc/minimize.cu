@@ -44,6 +44,9 @@ struct MinRpArgs {
   long long iters;   // at most this many moves in this launch
   int final_eval;    // evaluate |F| after the last move
   int R, NP, JP, unitw;
+  unsigned long long limit;  // of a barrier's wait, ns
+  long long stall_at;        // the barrier (counted from 0) that CTA stall_cta does not arrive at; -1: none
+  int stall_cta;
   TrapDev trap;
   SpeciesDev spc[IONTRAP_MAX_SPECIES];
 };
@@ -123,8 +126,8 @@ __global__ void __launch_bounds__(kMinT, 1) k_minimize_rp(const __grid_constant_
     ++arrived;
     __syncthreads();
     if (tid == 0) {
-      arrive_release(A.sync);
-      bad = !poll_wait<true>(A.sync, G * arrived, A.err, kWaitLimitNs);
+      if (!((int)blockIdx.x == A.stall_cta && arrived == A.stall_at + 1)) arrive_release(A.sync);
+      bad = !poll_wait<true>(A.sync, G * arrived, A.err, A.limit);
     }
     bad = __syncthreads_or(bad);
   };
@@ -521,6 +524,8 @@ cudaError_t launch_minimize(const StepArgs& s, void* scratch, bool cluster, int 
   A.dmax = reinterpret_cast<double*>(p + 256 + (size_t)s.n * sizeof(double2));
   A.dt = dt, A.dmaxlim = dmax, A.ftol = ftol, A.iters = iters, A.final_eval = final_eval;
   A.R = ions, A.NP = NP, A.JP = JP, A.unitw = s.unitw;
+  A.limit = s.wait_ns ? s.wait_ns : kWaitLimitNs;
+  A.stall_cta = s.stall_cta, A.stall_at = s.stall_on ? s.stall_step : -1;
   A.trap = s.trap;
   for (int k = 0; k < IONTRAP_MAX_SPECIES; ++k) A.spc[k] = s.spc[k];
   cudaError_t e = cudaMemsetAsync(A.sync, 0, sizeof(unsigned), st);

@@ -91,3 +91,32 @@ def test_a_withheld_last_arrival_is_a_timeout_too():
         assert e.value.code == it.IONTRAP_ETIMEOUT
         x, v, step, _ = it.iontrap_state(s.handle, n, accept=(it.IONTRAP_ETIMEOUT,))
         assert step == 0
+
+
+@pytest.mark.parametrize("cta,barrier", [(0, 0), (3, 7), (-1, 2)])
+def test_a_withheld_barrier_ends_a_minimisation(cta, barrier):
+    """The iterations' barriers on the grid (above 432 ions)."""
+    import paper_1907_10514_gb300 as it
+    n = 1030
+    x = iongen.gaussian_positions(n, 30e-6, seed=[n, 29])
+    p = it.make_params(None, Omega=iongen.OMEGA_RF, q=0.2, omega_z=2 * np.pi * 1e5, dt=iongen.rf_period_dt(iongen.OMEGA_RF),
+                       flags=it.IONTRAP_PSEUDO)
+    want = None
+    for stall in (False, True):
+        with it.Simulation([iongen.CA40], np.zeros(n, np.uint8), x, None, p) as s:
+            ctas = it.iontrap_test_step_kernel(s.handle)[1]
+            if not stall:  # beyond every launch: the limit alone changes nothing
+                it.iontrap_test_stall(s.handle, 200_000_000, cta % ctas, 1 << 40)
+                want = s.minimize(20, 5e-7, 0.0, 5e-8)
+                assert want[0] == 20
+                continue
+            it.iontrap_test_stall(s.handle, LIMIT_NS, cta % ctas, barrier)
+            t0 = time.perf_counter()
+            with pytest.raises(it.IonTrapError) as e:
+                s.minimize(20, 5e-7, 0.0, 5e-8)
+            assert e.value.code == it.IONTRAP_ETIMEOUT and time.perf_counter() - t0 < 1.0
+            with pytest.raises(it.IonTrapError) as e:  # sticky
+                s.minimize(20, 5e-7, 0.0, 5e-8)
+            assert e.value.code == it.IONTRAP_ETIMEOUT
+    with it.Simulation([iongen.CA40], np.zeros(n, np.uint8), x, None, p) as s:
+        assert s.minimize(20, 5e-7, 0.0, 5e-8) == want
