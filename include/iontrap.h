@@ -353,8 +353,9 @@ typedef struct {
                                  Up to 432 ions form 5 steps run on one thread-block
                                  cluster instead, with the same bits.
                                  The FP64 form supports 1 only; it sums every unordered pair
-                                 once in a layout that is a function of n, and threads,
-                                 ions_per_thread and jsplit do not change its results. */
+                                 once in a layout that is a function of n and the number of
+                                 SMs, and threads, ions_per_thread and jsplit do not change
+                                 its results.  Its scratch takes ~1.5 KB an ion for large n. */
     int32_t pdl;              /* 1: consecutive step kernels use programmatic dependent launch
                                  (default: 1 with fused = 0, whose epilogue then starts while
                                  the pairs are summed; otherwise 0, measured slower on GB300) */

@@ -64,8 +64,8 @@ cudaError_t launch_minimize(const StepArgs& s, void* scratch, bool cluster, int 
                             double dt, double dmax, double ftol, long long iters, int final_eval, int b,
                             cudaStream_t st);
 // pairs_f64.cu
-size_t f64_scratch_bytes(long long n, int sms);
-cudaError_t f64_prepare(long long n, int sms, void* scratch, cudaStream_t st, F64View* v);
+size_t f64_scratch_bytes(long long n, int sms, bool coulomb);
+cudaError_t f64_prepare(long long n, int sms, bool coulomb, void* scratch, cudaStream_t st, F64View* v);
 cudaError_t launch_f64(const StepArgs& a, const F64View& v, int nspecies, cudaStream_t st);
 // cluster_step.cu
 int rpc_ctas(long long n, int JP);
@@ -707,7 +707,8 @@ int alloc_scratch(iontrap* h) {
     return IONTRAP_EINVAL;
   // FP32 form: one 32-byte record per (split, ion); the row-persistent form also keeps
   // its part-major position copies there between the steps of a launch
-  size_t part = h->f64 ? f64_scratch_bytes(h->n, h->sms) : (size_t)splits * (size_t)h->n * 32;
+  const bool coulomb = !(h->p.flags & IONTRAP_COULOMB_OFF);
+  size_t part = h->f64 ? f64_scratch_bytes(h->n, h->sms, coulomb) : (size_t)splits * (size_t)h->n * 32;
   if (h->fused == 5) part = std::max(part, rp_scratch_bytes(h->rp.NP, h->rp.JP));
   const size_t cnt = (size_t)cdiv(h->n, iblock_ions(h));
   if (part > h->part_bytes) {
@@ -736,7 +737,7 @@ int alloc_scratch(iontrap* h) {
       if (cudaMemsetAsync(h->d_gsync, 0, bytes, h->stream) != cudaSuccess) return IONTRAP_ECUDA;
     }
   }
-  if (h->f64 && f64_prepare(h->n, h->sms, h->d_part, h->stream, &h->f64v) != cudaSuccess) return IONTRAP_ECUDA;
+  if (h->f64 && f64_prepare(h->n, h->sms, coulomb, h->d_part, h->stream, &h->f64v) != cudaSuccess) return IONTRAP_ECUDA;
   h->args.part = h->d_part;
   h->args.cnt = h->d_cnt;
   h->args.jsplit = (h->p.flags & IONTRAP_COULOMB_OFF) ? (int)std::min<int64_t>(h->n, 1 << 30)
@@ -1681,7 +1682,7 @@ int iontrap_estimate_bytes(int64_t n, int precision, int64_t* bytes) {
     T = tc.threads, I = tc.ions_per_thread, J = tc.jsplit, F = tc.fused;
   }
   const int64_t splits = F == 5 ? cdiv(n, kRpInitJsplit) : cdiv(n, J);
-  int64_t part = f64 ? (int64_t)f64_scratch_bytes(n, sms) : splits * n * 32;
+  int64_t part = f64 ? (int64_t)f64_scratch_bytes(n, sms, true) : splits * n * 32;
   if (F == 5 && rp_shape(n, f64, 0, sms, T, I, P, J, &rs))
     part = std::max<int64_t>(part, (int64_t)rp_scratch_bytes(rs.NP, rs.JP));
   const int64_t iblocks = F >= 4 ? cdiv(n, 256) : cdiv(n, (F == 3 ? 32 : (int64_t)T) * I);

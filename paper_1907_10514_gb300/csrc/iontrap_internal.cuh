@@ -101,12 +101,13 @@ struct BatchEns {
   SpeciesDev spc[IONTRAP_MAX_SPECIES];
 };
 
-// Scratch of an FP64 handle (pairs_f64.cu): its tables and slots, by offset from base, and the
-// shape of its pair line.
+// Scratch of an FP64 handle (pairs_f64.cu): its tables (of the first band) and slots, by offset
+// from base, and the shape of its pair line.
 struct F64View {
   void* base;
-  size_t off[9];
-  int I, rows, cols, warps;
+  size_t off[10];
+  size_t band_bytes;  // from a band's tables to the next's
+  int I, rows, cols, warps, bands;
 };
 
 // Result of a minimisation launch (minimize.cu).

@@ -14,11 +14,13 @@
 // its e^2 term in FP32.
 //
 // The triangle of (row block, column block, rotation) is one line of equal units, cut evenly
-// over all warps of the GPU by a table the host lays out once per handle.  The force-independent
+// over all warps of the GPU by a table the host lays out once per handle (above 16384 ions one per
+// band of kF64BandRows row blocks, each summed and folded into three sums per ion before the next:
+// the column slots would grow with n^2 and now take 1.5 KB an ion).  The force-independent
 // terms that are long FP64 chains (logarithm and square root of the noise, its sine and cosine,
 // cos(Omega t)) are units of the same line, so that they run beside the pairs.  Sums go to fixed
-// slots; k_finish_f64 adds an ion's slots in a fixed order, and integrates.  The result is a
-// function of n, the SM count and the inputs only.
+// slots; k_finish_f64 adds an ion's slots in a fixed order, and integrates after the last band.  The
+// result is a function of n, the SM count and the inputs only.
 //
 // Measured on GB300 (us per step, the form that summed every ordered pair with rsqrt(double)
 // against this one): n = 64: 19.3 -> 11.9, 321: 26.1 -> 16.4, 1000: 53.4 -> 29.3, 2500:
@@ -36,33 +38,43 @@ namespace it {
 // noise units.  A unit is one rotation of one (row block, column block) tile.
 struct F64Share {
   int a, c, k;     // first row block, column block, rotation
+  int tile;        // slot of that tile's column sums; the line's next tile has the next slot
   int units;       // rotations taken, crossing tiles and rows
   int flush;       // slot of the first row block's sums; the next row block's is flush + 1
   int first_main;  // the first tile is begun here (its column sums go to the main slot)
   int noise, nnoise;  // first noise unit and their number
 };
 
-struct F64Plan {
-  int I = 1, rows = 0, cols = 0, warps = 0, flushes = 0;
+struct F64Band {
+  int row0 = 0, rows = 0, flushes = 0;
   std::vector<F64Share> share;
   std::vector<int> row_flush;  // [rows + 1]: slots of a row block
   std::vector<int> col_extra;  // [cols + 1]: warps that continue a tile of a column block, below
   std::vector<int> extra;      // their numbers
 };
 
-// Device view: tables and slots in the handle's scratch.
+// Device view: a band's tables, and the slots, in the handle's scratch.
 struct F64Args {
   const F64Share* share;
   const int* row_flush;
   const int* col_extra;
   const int* extra;
   double* row_sum;   // [flushes][I][3][32]
-  double* col_sum;   // [rows][3][32 cols]: main column sums
+  double* col_sum;   // [tiles][3][32]: main column sums, the tiles of a row block side by side
   double* ext_sum;   // [warps][3][32]: column sums of continued tiles
   double* noise;     // [5][n16]: r1, r2, cos 1, sin 1, cos 2 (n16: n rounded up to 16)
   double* springs;   // [species][3] at the force time
-  int rows, cols, warps, nspecies, bath;
+  double* fold;      // [3][32 cols]: the sums of the bands before
+  int row0, rows;    // the band's row blocks
+  int cols, warps, nspecies, bath;
+  int first, last;   // of the bands
 };
+
+// The tile (row block row0 + r of I sub-blocks, column block c) of a band: row block r has
+// cols - (row0 + r) I of them.
+__host__ __device__ __forceinline__ int f64_tile_slot(int row0, int r, int I, int cols, int c) {
+  return r * (cols - row0 * I) - I * (r * (r - 1) / 2) + c - (row0 + r) * I;
+}
 
 constexpr int kF64Threads = 128;
 constexpr int kF64NoiseIons = 16;  // ions of a noise unit (32 lanes: two numbers each)
@@ -144,7 +156,7 @@ __global__ void __launch_bounds__(kF64Threads) k_pairs_f64(const __grid_constant
   // ions past n sit far away: r^-3 underflows to zero
   auto load = [&](long long i) { return i < n ? pos[i] : make_double4_32a(1e150, 1e150, 1e150, 0.0); };
   double* cj = &s_cj[wl][0][0];
-  int a = sh.a, c = sh.c, k = sh.k, flush = sh.flush;
+  int a = sh.a, c = sh.c, k = sh.k, tile = sh.tile, flush = sh.flush;
   int left = (A.trap.flags & IONTRAP_COULOMB_OFF) ? 0 : sh.units;
   bool main = sh.first_main != 0;
   double xi[I][3], zi[I], ai[I][3];
@@ -172,10 +184,10 @@ __global__ void __launch_bounds__(kF64Threads) k_pairs_f64(const __grid_constant
     left -= k1 - k;
     // lane l now holds the sums of column (l + k1) % 32
     const int col = (lane + k1) & 31;
-    double* out = main ? F.col_sum + ((long long)a * 3 * F.cols + c) * 32 + col : F.ext_sum + 96LL * w + col;
-    const long long stride = main ? 32LL * F.cols : 32;
+    double* out = (main ? F.col_sum + 96LL * tile : F.ext_sum + 96LL * w) + col;
+    ++tile;
 #pragma unroll
-    for (int q = 0; q < 3; ++q) __stcg(out + q * stride, aj[q]);
+    for (int q = 0; q < 3; ++q) __stcg(out + 32 * q, aj[q]);
     main = true;
     k = 0;
     if (++c == F.cols || left == 0) {
@@ -189,7 +201,7 @@ __global__ void __launch_bounds__(kF64Threads) k_pairs_f64(const __grid_constant
   }
 }
 
-// An ion's sums, then the rest of the step: a CTA per column block, kF64Slices warps per
+// An ion's sums over a band, and after the last one the rest of the step: a CTA per column block, kF64Slices warps per
 // component, each adding every kF64Slices-th slot of a kind with eight loads in flight (the
 // slots are ~60 at n = 4096: one warp's loads in turn would be the longest chain of the step).
 constexpr int kF64Slices = 4;
@@ -200,10 +212,11 @@ __global__ void __launch_bounds__(96 * kF64Slices)
   __shared__ double s_v[3][32];
   __shared__ double s_sum[kF64Slices][3][32];
   const int lane = threadIdx.x & 31, q = (threadIdx.x >> 5) % 3, z = threadIdx.x / 96;
-  const int c = blockIdx.x, a = c / I;
+  const int c = blockIdx.x, a = c / I, r = a - F.row0;  // r: the block's row in the band, if there
   const long long n = A.n, i = 32LL * c + lane;
   const long long ns = *A.step;
   const bool on = i < n, step = A.mode == MODE_STEP;
+  if (r < 0 && !F.last) return;
   if (!(A.trap.flags & IONTRAP_COULOMB_OFF)) {
     double S = 0.0;
     auto add = [&](auto slot, int m) {
@@ -223,14 +236,27 @@ __global__ void __launch_bounds__(96 * kF64Slices)
       for (int k = 0; k < 7; ++k) t[k & 3] += g[k];
       S += (t[0] + t[1]) + (t[2] + t[3]);
     };
-    const int f0 = F.row_flush[a], e0 = F.col_extra[c];
+    const bool row = r >= 0 && r < F.rows;
+    const int f0 = row ? F.row_flush[r] : 0, e0 = F.col_extra[c];
     add([&](int u) { return F.row_sum + (((f0 + u) * (long long)I + (c - a * I)) * 3 + q) * 32 + lane; },
-        F.row_flush[a + 1] - f0);
-    add([&](int u) { return F.col_sum + ((3LL * u + q) * F.cols + c) * 32 + lane; }, a + 1);
+        row ? F.row_flush[r + 1] - f0 : 0);
+    add([&](int u) { return F.col_sum + 96LL * f64_tile_slot(F.row0, u, I, F.cols, c) + 32 * q + lane; },
+        max(0, min(r + 1, F.rows)));
     add([&](int u) { return F.ext_sum + 96LL * F.extra[e0 + u] + 32 * q + lane; }, F.col_extra[c + 1] - e0);
     s_sum[z][q][lane] = S;
   } else {
     s_sum[z][q][lane] = 0.0;
+  }
+  double* fold = F.fold + 32LL * F.cols * q + i;
+  if (!F.last) {
+    __syncthreads();
+    if (z == 0) {
+      double S = s_sum[0][q][lane];
+#pragma unroll
+      for (int k = 1; k < kF64Slices; ++k) S += s_sum[k][q][lane];
+      __stcg(fold, F.first ? S : __ldcg(fold) + S);
+    }
+    return;
   }
   const SpeciesDev& sd = A.spc[on ? A.sp[i] : 0];
   double v = 0.0, vd = 0.0, xf = 0.0, ext = 0.0;
@@ -248,6 +274,7 @@ __global__ void __launch_bounds__(96 * kF64Slices)
     double S = s_sum[0][q][lane];
 #pragma unroll
     for (int k = 1; k < kF64Slices; ++k) S += s_sum[k][q][lane];
+    if (!F.first) S += __ldcg(fold);
     if (A.mode == MODE_FORCES) {
       A.out[q * n + i] = sd.coul * S;
     } else {
@@ -295,80 +322,104 @@ static int f64_rows(long long n) { return n <= 2048 ? 1 : n <= 4096 ? 2 : n <= 8
 // n = 64: 11.5 11.9 12.4 15.4; 321: 17.8 16.4 15.9 17.8; 1000: 29.3 29.3 29.3 29.3).
 constexpr long long kF64NoiseCost = 5;  // of a noise unit, in rotations of one sub-block (16 FP64 instructions)
 constexpr long long kF64MinCost = 3;
+// Row blocks of a band: all of them up to 16384 ions.  A further band costs the end of its launch,
+// where warps finish at different times, and the fold (all row blocks in one band / in bands, and
+// the handle's memory: n = 32768: 15.09 / 15.13 ms per step, 116 / 53 MB; 100000: 140.1 / 140.4 ms,
+// 967 / 171 MB).
+constexpr int kF64BandRows = 64;
 
-static F64Plan f64_plan(long long n, int sms) {
-  F64Plan P;
-  P.I = f64_rows(n);
-  P.cols = (int)((n + 31) / 32);
-  P.rows = (P.cols + P.I - 1) / P.I;
-  const int m = (int)((n + kF64NoiseIons - 1) / kF64NoiseIons), units = 2 * m + 1;
-  // cost of rotation k of a tile at distance d = c - a I from its row block
-  auto cost = [&](int d, int k) -> long long {
-    return std::min(d, P.I) + (d < P.I && k >= 1 && k <= 16 ? 1 : 0);
-  };
-  auto tile_cost = [&](int d) -> long long { return 32LL * std::min(d, P.I) + (d < P.I ? 16 : 0); };
-  long long pair_total = 0;
-  for (int a = 0; a < P.rows; ++a)
-    for (int c = a * P.I; c < P.cols; ++c) {
-      const int d = c - a * P.I;
-      if (d >= P.I) {
-        pair_total += tile_cost(d) * (P.cols - c);
-        break;
+// The shape of n ions' bands; without the pair term there are noise units only.
+struct F64Shape {
+  int I, rows, cols, bands, units, warps;
+  long long tile_cost(int d) const { return 32LL * std::min(d, I) + (d < I ? 16 : 0); }  // d: columns from its row block
+  int band_rows(int b) const { return std::min(kF64BandRows, rows - b * kF64BandRows); }
+  long long cost(int b) const {
+    long long t = b == 0 ? kF64NoiseCost * units : 0;
+    for (int a = b * kF64BandRows; a < b * kF64BandRows + band_rows(b); ++a)
+      for (int c = a * I; c < cols; ++c) {
+        const int d = c - a * I;
+        if (d >= I) {
+          t += tile_cost(d) * (cols - c);
+          break;
+        }
+        t += tile_cost(d);
       }
-      pair_total += tile_cost(d);
-    }
-  const long long total = pair_total + kF64NoiseCost * units;
-  P.warps = (int)std::max<long long>(1, std::min<long long>(8LL * sms, total / kF64MinCost));
-  P.share.resize(P.warps);
-  P.row_flush.assign(P.rows + 1, 0);
-  std::vector<std::vector<int>> extra(P.cols);
-  int a = 0, c = 0, k = 0;
+    return t;
+  }
+};
+
+static F64Shape f64_shape(long long n, int sms, bool coulomb) {
+  F64Shape S{};
+  S.I = f64_rows(n);
+  S.cols = (int)((n + 31) / 32);
+  S.rows = coulomb ? (S.cols + S.I - 1) / S.I : 0;
+  S.bands = std::max(1, (S.rows + kF64BandRows - 1) / kF64BandRows);
+  S.units = 2 * (int)((n + kF64NoiseIons - 1) / kF64NoiseIons) + 1;
+  S.warps = (int)std::max<long long>(1, std::min<long long>(8LL * sms, S.cost(0) / kF64MinCost));
+  return S;
+}
+
+static F64Band f64_band(const F64Shape& S, int b) {
+  F64Band B;
+  B.row0 = b * kF64BandRows, B.rows = S.band_rows(b);
+  const int I = S.I, cols = S.cols, end_row = B.row0 + B.rows, units = b == 0 ? S.units : 0;
+  // cost of rotation k of a tile at distance d = c - a I from its row block
+  auto cost = [&](int d, int k) -> long long { return std::min(d, I) + (d < I && k >= 1 && k <= 16 ? 1 : 0); };
+  const long long total = S.cost(b);
+  B.share.resize(S.warps);
+  B.row_flush.assign(B.rows + 1, 0);
+  std::vector<std::vector<int>> extra(cols);
+  int a = B.row0, c = a * I, k = 0;
   long long done = 0;
   int u = 0;
-  for (int w = 0; w < P.warps; ++w) {
+  for (int w = 0; w < S.warps; ++w) {
     // the cost line up to this warp's end; noise first (it is the longest chain)
-    const long long end = total * (w + 1) / P.warps;
-    F64Share& s = P.share[w];
+    const long long end = total * (w + 1) / S.warps;
+    F64Share& s = B.share[w];
     s.noise = u;
     while (u < units && done < end) ++u, done += kF64NoiseCost;
     s.nnoise = u - s.noise;
-    s.a = a, s.c = c, s.k = k, s.units = 0, s.flush = P.flushes, s.first_main = k == 0;
-    if (a < P.rows && (done < end || w + 1 == P.warps) && k != 0) extra[c].push_back(w);
+    s.a = a, s.c = c, s.k = k, s.tile = f64_tile_slot(B.row0, a - B.row0, I, cols, c), s.units = 0, s.flush = B.flushes, s.first_main = k == 0;
+    const bool last = w + 1 == S.warps;
+    if (a < end_row && (done < end || last) && k != 0) extra[c].push_back(w);
     bool open = false;
-    const bool last = w + 1 == P.warps;
-    while (a < P.rows && (done < end || last)) {
-      if (!open) open = true;
-      const int d = c - a * P.I;
-      if (k == 0 && d >= P.I && !last && done + tile_cost(d) <= end) {  // whole tiles at once
-        s.units += 32, done += tile_cost(d), k = 32;
+    while (a < end_row && (done < end || last)) {
+      open = true;
+      const int d = c - a * I;
+      if (k == 0 && d >= I && !last && done + S.tile_cost(d) <= end) {  // whole tiles at once
+        const long long m = std::min<long long>(cols - c, (end - done) / S.tile_cost(d));
+        s.units += 32 * (int)m, done += m * S.tile_cost(d), k = 32, c += (int)m - 1;
       } else {
         ++s.units, done += cost(d, k), ++k;
       }
       if (k == 32) {
         k = 0;
-        if (++c == P.cols) {
-          P.row_flush[a + 1] = ++P.flushes;
+        if (++c == cols) {
+          ++B.flushes;
           open = false;
-          ++a, c = a * P.I;
+          ++a, c = a * I;
+          B.row_flush[a - B.row0] = B.flushes;
         }
       }
     }
-    if (open) ++P.flushes, P.row_flush[a + 1] = P.flushes;
+    if (open) ++B.flushes;
   }
-  P.col_extra.assign(P.cols + 1, 0);
-  for (int q = 0; q < P.cols; ++q) {
-    for (int w : extra[q]) P.extra.push_back(w);
-    P.col_extra[q + 1] = (int)P.extra.size();
+  B.col_extra.assign(cols + 1, 0);
+  for (int q = 0; q < cols; ++q) {
+    for (int w : extra[q]) B.extra.push_back(w);
+    B.col_extra[q + 1] = (int)B.extra.size();
   }
-  return P;
+  return B;
 }
 
-// Scratch layout in bytes: tables, then slots.
+// Scratch layout in bytes: the bands' tables, then the slots that they share.  Sizes follow from
+// the shape: a warp leaves one row block's sums open at most and continues one tile.
 struct F64Layout {
-  size_t share, row_flush, col_extra, extra, row_sum, col_sum, ext_sum, noise, springs, bytes;
+  size_t share, row_flush, col_extra, extra, band;  // a band's tables, and the bytes from one to the next
+  size_t row_sum, col_sum, ext_sum, noise, springs, fold, bytes;
 };
 
-static F64Layout f64_layout(const F64Plan& P, long long n) {
+static F64Layout f64_layout(const F64Shape& S, long long n) {
   F64Layout L{};
   size_t at = 0;
   auto take = [&](size_t bytes) {
@@ -376,35 +427,49 @@ static F64Layout f64_layout(const F64Plan& P, long long n) {
     at += (bytes + 255) / 256 * 256;
     return p;
   };
-  L.share = take(P.share.size() * sizeof(F64Share));
-  L.row_flush = take(P.row_flush.size() * sizeof(int));
-  L.col_extra = take(P.col_extra.size() * sizeof(int));
-  L.extra = take(std::max<size_t>(1, P.extra.size()) * sizeof(int));
-  L.row_sum = take((size_t)P.flushes * P.I * 96 * sizeof(double));
-  L.col_sum = take((size_t)P.rows * 96 * P.cols * sizeof(double));
-  L.ext_sum = take((size_t)P.warps * 96 * sizeof(double));
+  const int rows = S.band_rows(0);
+  const size_t tiles = rows ? (size_t)(f64_tile_slot(0, rows - 1, S.I, S.cols, S.cols - 1) + 1) : 0;
+  L.share = take(S.warps * sizeof(F64Share));
+  L.row_flush = take((rows + 1) * sizeof(int));
+  L.col_extra = take((S.cols + 1) * sizeof(int));
+  L.extra = take(S.warps * sizeof(int));
+  L.band = at;
+  at *= S.bands;
+  const size_t warps = S.rows ? S.warps : 0;
+  L.row_sum = take((warps + rows) * S.I * 96 * sizeof(double));
+  L.col_sum = take(tiles * 96 * sizeof(double));
+  L.ext_sum = take(warps * 96 * sizeof(double));
   L.noise = take(5 * (size_t)((n + 15) / 16 * 16) * sizeof(double));
   L.springs = take(3 * IONTRAP_MAX_SPECIES * sizeof(double));
+  L.fold = take(S.bands > 1 ? 96 * (size_t)S.cols * sizeof(double) : 0);
   L.bytes = at;
   return L;
 }
 
-size_t f64_scratch_bytes(long long n, int sms) { return f64_layout(f64_plan(n, sms), n).bytes; }
+size_t f64_scratch_bytes(long long n, int sms, bool coulomb) {
+  return f64_layout(f64_shape(n, sms, coulomb), n).bytes;
+}
 
 // Lay out a handle's scratch: its tables are written (synchronously, the host copy goes away)
 // and *v is what the launches need.
-cudaError_t f64_prepare(long long n, int sms, void* scratch, cudaStream_t st, F64View* v) {
-  const F64Plan P = f64_plan(n, sms);
-  const F64Layout L = f64_layout(P, n);
+cudaError_t f64_prepare(long long n, int sms, bool coulomb, void* scratch, cudaStream_t st, F64View* v) {
+  const F64Shape S = f64_shape(n, sms, coulomb);
+  const F64Layout L = f64_layout(S, n);
   v->base = scratch;
-  v->I = P.I, v->rows = P.rows, v->cols = P.cols, v->warps = P.warps;
-  const size_t off[9] = {L.share, L.row_flush, L.col_extra, L.extra, L.row_sum, L.col_sum, L.ext_sum, L.noise, L.springs};
+  v->I = S.I, v->rows = S.rows, v->cols = S.cols, v->warps = S.warps, v->bands = S.bands;
+  const size_t off[10] = {L.share, L.row_flush, L.col_extra, L.extra, L.row_sum,
+                          L.col_sum, L.ext_sum, L.noise, L.springs, L.fold};
   std::memcpy(v->off, off, sizeof(off));
-  std::vector<unsigned char> h(L.row_sum);
-  std::memcpy(h.data() + L.share, P.share.data(), P.share.size() * sizeof(F64Share));
-  std::memcpy(h.data() + L.row_flush, P.row_flush.data(), P.row_flush.size() * sizeof(int));
-  std::memcpy(h.data() + L.col_extra, P.col_extra.data(), P.col_extra.size() * sizeof(int));
-  std::memcpy(h.data() + L.extra, P.extra.data(), P.extra.size() * sizeof(int));
+  v->band_bytes = L.band;
+  std::vector<unsigned char> h(L.band * S.bands);
+  for (int b = 0; b < S.bands; ++b) {
+    const F64Band B = f64_band(S, b);
+    unsigned char* t = h.data() + L.band * b;
+    std::memcpy(t + L.share, B.share.data(), B.share.size() * sizeof(F64Share));
+    std::memcpy(t + L.row_flush, B.row_flush.data(), B.row_flush.size() * sizeof(int));
+    std::memcpy(t + L.col_extra, B.col_extra.data(), B.col_extra.size() * sizeof(int));
+    if (!B.extra.empty()) std::memcpy(t + L.extra, B.extra.data(), B.extra.size() * sizeof(int));
+  }
   const cudaError_t e = cudaMemcpyAsync(scratch, h.data(), h.size(), cudaMemcpyHostToDevice, st);
   return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
 }
@@ -412,16 +477,13 @@ cudaError_t f64_prepare(long long n, int sms, void* scratch, cudaStream_t st, F6
 cudaError_t launch_f64(const StepArgs& a, const F64View& v, int nspecies, cudaStream_t st) {
   char* b = static_cast<char*>(v.base);
   F64Args F{};
-  F.share = reinterpret_cast<const F64Share*>(b + v.off[0]);
-  F.row_flush = reinterpret_cast<const int*>(b + v.off[1]);
-  F.col_extra = reinterpret_cast<const int*>(b + v.off[2]);
-  F.extra = reinterpret_cast<const int*>(b + v.off[3]);
   F.row_sum = reinterpret_cast<double*>(b + v.off[4]);
   F.col_sum = reinterpret_cast<double*>(b + v.off[5]);
   F.ext_sum = reinterpret_cast<double*>(b + v.off[6]);
   F.noise = reinterpret_cast<double*>(b + v.off[7]);
   F.springs = reinterpret_cast<double*>(b + v.off[8]);
-  F.rows = v.rows, F.cols = v.cols, F.warps = v.warps, F.nspecies = nspecies;
+  F.fold = reinterpret_cast<double*>(b + v.off[9]);
+  F.cols = v.cols, F.warps = v.warps, F.nspecies = nspecies;
   for (int s = 0; s < nspecies; ++s) F.bath |= a.spc[s].sigma > 0.0;
   const void* pairs = nullptr;
   const void* finish = nullptr;
@@ -434,8 +496,18 @@ cudaError_t launch_f64(const StepArgs& a, const F64View& v, int nspecies, cudaSt
   StepArgs ac = a;
   void* params[] = {&ac, &F};
   const int per = kF64Threads / 32;
-  cudaError_t e = cudaLaunchKernel(pairs, dim3((unsigned)((v.warps + per - 1) / per)), dim3(kF64Threads), params, 0, st);
-  if (e == cudaSuccess) e = cudaLaunchKernel(finish, dim3((unsigned)v.cols), dim3(96 * kF64Slices), params, 0, st);
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k < v.bands && e == cudaSuccess; ++k) {
+    char* t = b + v.band_bytes * k;
+    F.share = reinterpret_cast<const F64Share*>(t + v.off[0]);
+    F.row_flush = reinterpret_cast<const int*>(t + v.off[1]);
+    F.col_extra = reinterpret_cast<const int*>(t + v.off[2]);
+    F.extra = reinterpret_cast<const int*>(t + v.off[3]);
+    F.row0 = k * kF64BandRows, F.rows = std::min(kF64BandRows, v.rows - F.row0);
+    F.first = k == 0, F.last = k + 1 == v.bands;
+    e = cudaLaunchKernel(pairs, dim3((unsigned)((v.warps + per - 1) / per)), dim3(kF64Threads), params, 0, st);
+    if (e == cudaSuccess) e = cudaLaunchKernel(finish, dim3((unsigned)v.cols), dim3(96 * kF64Slices), params, 0, st);
+  }
   return e;
 }
 
