@@ -277,7 +277,7 @@ __device__ __forceinline__ double square21(double y) {
   return __longlong_as_double((long long)((unsigned long long)(2u * e - 1023u + up) << 52 | f));
 }
 
-// What r^-1, r^-2 and r^-3 are built from: y, the 21-bit approximation of r2^(-1/2), y^2 exactly,
+// What r^-3 is built from: y, the 21-bit approximation of r2^(-1/2), y^2 exactly,
 // e = 1 - r2 y^2 and e^2, of which 20 bits count, without the FP64 pipe (|e| below 2^-18, or
 // zero, or not a number; tiny e gives 0).
 struct InvParts {
@@ -307,11 +307,6 @@ __device__ __forceinline__ double inv_cube(double r2, const InvParts& p) {
   return __double2hiint(r2) == 0x7ff00000 ? 0.0 : s;
 }
 __device__ __forceinline__ double inv_cube(double r2) { return inv_cube(r2, inv_parts(r2)); }
-
-// r^-2: y^2 / (1 - e).
-__device__ __forceinline__ double inv_square(const InvParts& p) {
-  return __fma_rn(p.y2, p.e + widen_normal(p.e2), p.y2);
-}
 
 // ------------------------------------------------------------------ FP32 pair terms
 // d = x_j - x_i from hi/lo pairs, with the i side held negated in registers:

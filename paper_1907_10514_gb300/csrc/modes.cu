@@ -257,19 +257,46 @@ struct HessArgs {
 
 // A CTA per ion i, a thread per j: the row's off-diagonal blocks, and the diagonal block
 // from their sum (fixed order: j by threads, then a tree), plus the trap springs M_i k_a, over
-// M_i.  A pair block is kq (delta_ab r^-3 - 3 r_a r_b r^-5), symmetric, from r^-2 and r^-3
-// without a division or a root: ~36 FP64 instructions a pair, where eighteen divisions in
-// two kernels took ~500 (n = 300, with the copy to the host: 251 -> 79 us a call).
+// M_i.  A pair block is kq (delta_ab r^-3 - 3 r_a r_b r^-5), symmetric, from r^-3 and r^-5
+// without a division or a root: ~52 FP64 instructions a pair, where eighteen divisions in
+// two kernels took ~500 (n = 300, with the copy to the host: 251 -> 83 us a call).  Fourteen of them
+// carry the rounding of r^2 along (80 us without): a block's largest error over its largest entry
+// is 2.0e-16 in the mean, 2.5e-16 with a rounded r^2 and r^-5 = r^-3 r^-2, 2.7e-16 with divisions.
 constexpr int kHessThreads = 128;
+
+// a + b and what the rounding left, for a, b >= 0 (the larger exponent first, compared as integers).
+__device__ __forceinline__ double sum2(double a, double b, double& lo) {
+  const bool less = __double2hiint(a) < __double2hiint(b);
+  const double u = less ? b : a, v = less ? a : b, s = u + v;
+  lo = v - (s - u);
+  return s;
+}
+
+// r^-3 and r^-5 of a difference: y = r^-1 to 21 bits, e = 1 - r^2 y^2, y^3 (1 - e)^(-3/2) and
+// y^5 (1 - e)^(-5/2) to e^2 (|e| < 2^-19).  A rounding of r^2 would count 2.5 times in r^-5: e takes
+// it along.
+__device__ __forceinline__ void inv_cube_fifth(const double (&r)[3], double& r3, double& r5) {
+  double p[3], lo[3], l1, l2;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) p[c] = __dmul_rn(r[c], r[c]), lo[c] = __fma_rn(r[c], r[c], -p[c]);
+  const double r2 = sum2(sum2(p[0], p[1], l1), p[2], l2);
+  const double rest = ((lo[0] + lo[1]) + (lo[2] + l1)) + l2;
+  const double y = rsqrt_approx_f64(r2), y2 = square21(y);
+  const double e = __fma_rn(-rest, y2, __fma_rn(-r2, y2, 1.0));
+  const double y3 = y2 * y, y5 = y3 * y2;
+  r3 = __fma_rn(y3, e * __fma_rn(1.875, e, 1.5), y3);
+  r5 = __fma_rn(y5, e * __fma_rn(4.375, e, 2.5), y5);
+}
 
 __global__ void __launch_bounds__(kHessThreads) k_hessian(const __grid_constant__ HessArgs A) {
   __shared__ double sh[6][kHessThreads];
-  __shared__ double s_w[IONTRAP_MAX_SPECIES], s_kq[IONTRAP_MAX_SPECIES];
+  __shared__ double s_w[IONTRAP_MAX_SPECIES], s_kq[IONTRAP_MAX_SPECIES], s_kq3[IONTRAP_MAX_SPECIES];
   const long long n = A.n, m = 3 * n;
   const int i = blockIdx.x, tid = threadIdx.x, si = A.sp[i];
   if (tid < IONTRAP_MAX_SPECIES) {
     s_w[tid] = 1.0 / sqrt(A.spc[si].mass * A.spc[tid].mass);
     s_kq[tid] = A.ke2 * A.spc[si].z * A.spc[tid].z;
+    s_kq3[tid] = 3.0 * s_kq[tid];
   }
   __syncthreads();
   const double xi[3] = {A.x[i], A.x[n + i], A.x[2 * n + i]};
@@ -280,10 +307,9 @@ __global__ void __launch_bounds__(kHessThreads) k_hessian(const __grid_constant_
 #pragma unroll
     for (int c = 0; c < 3; ++c) r[c] = xi[c] - A.x[c * n + j];
     const int sj = A.sp[j];
-    const double r2 = __fma_rn(r[0], r[0], __fma_rn(r[1], r[1], r[2] * r[2]));
-    const InvParts p = inv_parts(r2);
-    const double k3 = s_kq[sj] * inv_cube(r2, p);
-    const double k5 = 3.0 * k3 * inv_square(p);
+    double k3, k5;
+    inv_cube_fifth(r, k3, k5);
+    k3 *= s_kq[sj], k5 *= s_kq3[sj];
     const double t[3] = {r[0] * k5, r[1] * k5, r[2] * k5};
     const double b[6] = {__fma_rn(-t[0], r[0], k3), __fma_rn(-t[1], r[1], k3), __fma_rn(-t[2], r[2], k3),
                          -t[0] * r[1], -t[0] * r[2], -t[1] * r[2]};
