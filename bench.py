@@ -523,8 +523,8 @@ def modes_measurements(it, stream):
         wall = time.perf_counter() - t0
     out["minimize_crystal_n1024"] = {"iterations": iters, "seconds": wall, "us_per_iteration": 1e6 * wall / max(iters, 1),
                                      "force_norm_over_scale": fn / fscale,
-                                     "note": "FP32 pair kernel + 3 reduction/update kernels per iteration, "
-                                             "host check every 64 iterations"}
+                                     "note": "up to 1000 iterations per cooperative launch (FP32 pairs, FP64 "
+                                             "update), a look at the result after each launch"}
     nh = 2048
     xh = iongen.gaussian_positions(nh, 80e-6, seed=6)
     with it.Simulation([iongen.CA40], np.zeros(nh, np.uint8), xh, None, p, stream=stream) as s:

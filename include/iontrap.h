@@ -350,8 +350,13 @@ typedef struct {
                                     IONTRAP_COULOMB_OFF.
                                  Form 5 gives results within the FP32 tolerances of the other
                                  forms, bitwise reproducible for a given shape.
-                                 Up to 432 ions form 5 steps run on one thread-block
-                                 cluster instead, with the same bits.
+                                 Two kernels step small and middling n in this form instead,
+                                 with the same bits: one thread-block cluster up to 168 ions
+                                 (432 with threads = 512), above that and up to 2176 ions, with
+                                 threads = 256 and parts of at most 128 j, the grid with
+                                 positions that carry the step's tag, without the counter and
+                                 the copies.  Handles by default take the cluster up to 168
+                                 ions, the tagged grid up to 2047, the counter above.
                                  The FP64 form supports 1 only; it sums every unordered pair
                                  once in a layout that is a function of n and the number of
                                  SMs, and threads, ions_per_thread and jsplit do not change
@@ -494,6 +499,10 @@ int iontrap_test_step_kernel(const iontrap_t *h, int32_t *kernel, int32_t *ctas)
  * (start after the grid dependency wait, end of the pair loop, start of the fused
  * epilogue or 0, end of the fused epilogue or 0), then 2 per epilogue-kernel CTA (start,
  * end) when the configuration is not fused.  *n_force and *n_epi receive the counts.
+ * Form 5 handles whose steps run on one cluster (up to 168 ions by default) are traced on the
+ * grid instead, where marks are per CTA of `jsplit` ions: the marks are not those of the kernel
+ * that iontrap_step launches there (iontrap_test_step_kernel tells); the FP64 form and its
+ * kernels have no marks (zeros).
  * Synchronous; EINVAL if cap is too small. */
 int iontrap_trace_step(iontrap_t *h, unsigned long long *marks, int64_t cap, int64_t *n_force, int64_t *n_epi);
 

@@ -390,10 +390,12 @@ size_t rpc_smem_bytes(int Rc, int NPe, int JP, long long K) {
 //   n = 16: 2.84 / 1.15 1.07 - -      64: 3.30 / - 1.26 1.21 1.23    100: 4.97 / - 1.61 1.57 1.43
 //   128: 5.69 / - 2.05 1.73 1.53     200: 4.09 / - - 2.50 2.14       256: 4.13 / - - 3.06 2.58
 //   400: 3.49 / - - - 3.10           512: 3.51 / - - - 4.1
-// Above 168 ions most shapes are stepped by tagged_step.cu instead.
+// Above 168 ions shapes of 8 warps are stepped by tagged_step.cu instead.
+static int rpc_entries(long long n, int C) { return (int)(((n + 3) / 4 + C - 1) / C * 4); }
 int rpc_ctas(long long n, int JP) {
   if (JP > kSeg || n > kRpcMaxN) return 0;
-  return n < 13 ? 1 : n < 29 ? 4 : n <= 84 ? 8 : 16;
+  const int C = n < 13 ? 1 : n < 29 ? 4 : n <= 84 ? 8 : 16;
+  return rpc_entries(n, C) <= kRpcMaxRc ? C : 0;  // three owner threads an entry
 }
 
 cudaError_t launch_rpc(const StepArgs& a, int nspecies, int C, int JP, long long K, cudaStream_t st) {
@@ -402,7 +404,7 @@ cudaError_t launch_rpc(const StepArgs& a, int nspecies, int C, int JP, long long
   P.JP = JP;
   P.nspecies = nspecies;
   P.NPe = (int)((a.n + JP - 1) / JP);
-  P.Rc = (int)(((a.n + 3) / 4 + C - 1) / C * 4);
+  P.Rc = rpc_entries(a.n, C);
   const size_t smem = rpc_smem_bytes(P.Rc, P.NPe, JP, K);
   const auto fn = a.unitw ? k_step_f32_rpc<true> : k_step_f32_rpc<false>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);

@@ -50,7 +50,8 @@ struct ForcesArgs {
 // I ions per lane: 1, or 2 packed.  M: CTAs of eight warps that the registers leave room for, at
 // least.  Without that bound the compiler took 158 for the pair loop written in stages of 16 j and
 // two CTAs of five warps shared an SM (n = 5000: 28.5 us a call, 24.6 with M = 1 and 95 registers);
-// 64 registers (M = 4) take stages of 4 j.
+// 64 registers (M = 4) take stages of 4 j, and with two ions and unit charges still one spilled word,
+// which the fourth CTA outweighs (n = 7000: 45.9 -> 39.2 us).
 template <int I, bool UNITW, int M>
 __global__ void __launch_bounds__(32 * kMaxChunks, M) k_forces_cluster(const __grid_constant__ ForcesArgs A) {
   constexpr int kBlockIons = 32 * I, kStage = M == 1 ? 16 : 4;
