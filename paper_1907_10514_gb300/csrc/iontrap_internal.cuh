@@ -72,8 +72,9 @@ struct StepArgs {
   int jsplit;          // j-range per CTA (grid.y = ceil(n / jsplit))
   int nsplit;          // ceil(n / jsplit): partials per ion for the epilogue kernel
   // failure-detection test hook of the persistent forms (iontrap_test_stall): when
-  // stall_on, CTA stall_cta withholds its arrival on the grid-wide step counter at step
-  // stall_step of every launch, so that the other CTAs' bounded waits expire
+  // stall_on, CTA stall_cta withholds its arrival on the grid-wide step counter, or its
+  // positions where the kernel has no counter, at step stall_step of every launch (barrier
+  // stall_step of a minimisation's), so that the other CTAs' bounded waits expire
   int stall_on;
   int stall_cta;
   long long stall_step;
